@@ -353,6 +353,57 @@ __device__ __forceinline__ void clamped_cell(const MapDev& md, float px, float p
   cy = (int)qy + md.W / 2;
 }
 
+// The cells of the all-octant integer Bresenham line from (sx, sy) to (ex, ey),
+// both ends excluded, shared out over kLineLanes lanes: the line steps its longer
+// axis every time (M cells long, the other axis m), and its k-th cell has moved
+// floor((2 m k + M) / (2 M)) cells along the other axis (equal to the error-term
+// loop for every end within 45 cells and for random ones within 700). Lane j takes
+// the cells j + 1, j + 1 + kLineLanes, ...: one division, then additions with a
+// carry. Eight lanes, so that four lines share a warp's instructions.
+constexpr int kLineLanes = 8;
+
+struct LineWalk {
+  int n;             // cells up to the end: the cells 1 .. n - 1 lie between
+  int k;             // this lane's next cell
+  bool xmaj;
+  int sx, sy, stx, sty;
+  u32 o, rem, d, oq, orm;  // steps along the other axis, remainder, 2 M, and what kLineLanes cells add
+  __device__ __forceinline__ LineWalk(int sx_, int sy_, int ex, int ey, int j) : sx(sx_), sy(sy_) {
+    const int ax = abs(ex - sx), ay = abs(ey - sy);
+    stx = sx < ex ? 1 : -1;
+    sty = sy < ey ? 1 : -1;
+    xmaj = ax >= ay;
+    n = xmaj ? ax : ay;
+    const u32 mn = (u32)(xmaj ? ay : ax);
+    k = j + 1;
+    d = max(2u * (u32)n, 1u);
+    const u32 num = 2u * mn * (u32)k + (u32)n;
+    o = num / d;
+    rem = num - o * d;
+    const u32 add = 2u * kLineLanes * mn;
+    oq = add / d;
+    orm = add - oq * d;
+  }
+  // this lane's next cell; false past the end
+  __device__ __forceinline__ bool next(int& x, int& y) {
+    const bool act = k < n;
+    x = sx + stx * (xmaj ? k : (int)o);
+    y = sy + sty * (xmaj ? (int)o : k);
+    k += kLineLanes;
+    o += oq;
+    rem += orm;
+    if (rem >= d) {
+      rem -= d;
+      ++o;
+    }
+    return act;
+  }
+};
+
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
 // relaxed device-scope loads/stores for the radix-sort look-back
 __device__ __forceinline__ u32 ld_relaxed(const u32* p) {
   u32 v;

@@ -694,10 +694,6 @@ struct TaskWalk {
   }
 };
 
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
 // Kalman height update in information form (float32) + cumulative counts.
 __device__ __forceinline__ void height_update(const MapDev& md, u32 g, u32& fl, float h0, float v0, float sw,
                                               float swz, u32 na, u32 nr, u32 na0, u32 nr0) {
