@@ -8,21 +8,22 @@
 // sequences, so the result does not depend on the launch.
 //
 // PCA: per map, over the cells where the layer is observed,
-//   1. mean: blocks take fixed cell ranges, threads take channels; the block
-//      sums (float32) are added in block order in float64;
-//   2. covariance of (f - mean): blocks take fixed cell ranges and stage 32
-//      centred rows at a time in shared memory; each thread accumulates a
-//      T x T tile of the C x C matrix with float32 FMAs; the partial matrices
-//      are added in block order in float64;
+//   1. mean: blocks take fixed cell ranges, warps take rows with their lanes over
+//      the channels; the block sums (float32) are added in a fixed order in float64;
+//   2. covariance of (f - mean): blocks take fixed cell ranges and stage centred
+//      rows in shared memory; each thread accumulates an 8 x 8 tile of the upper
+//      triangle of the C x C matrix with float32 FMAs; the partial matrices are
+//      added in a fixed order in float64;
 //   3. eigenvectors: one block runs cyclic Jacobi sweeps (round-robin pairs,
 //      C/2 disjoint rotations at a time) in float32 shared memory until the
 //      off-diagonal mass is at the float32 rounding level of the matrix
 //      (at most 20 sweeps), then sorts the
 //      eigenvalues and signs each kept vector so that its largest-magnitude
 //      component is positive;
-//   4. projection of every observed cell on the kept vectors.
+//   4. projection of every observed cell on the kept vectors, four lanes a cell.
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "mem_host.h"
@@ -92,7 +93,8 @@ __global__ void __launch_bounds__(256) k_normals(MapDev md, int map, int rx, int
 // PCA
 
 constexpr int kPcaMaxC = 128;      // channels of a PCA input layer
-constexpr int kPcaRows = 32;       // centred rows staged at a time by the covariance blocks
+constexpr int kPcaRows = 64;       // centred rows staged at a time by the covariance blocks
+constexpr int kPcaBlocks = 2;      // blocks per SM of the mean and covariance kernels
 constexpr int kPcaMaxComp = 8;
 
 struct PcaArgs {
@@ -101,7 +103,7 @@ struct PcaArgs {
   int S, dtype;
   u32 obs_bit;
   double* mean_part;  // [blocks][C + 1] (sums, then the count)
-  float* cov_part;    // [blocks][C][C]
+  float* cov_part;    // [blocks][64][tiles] (element of the tile, tile)
   float* mean;        // [C]
   float* cov;         // [C][C]
   float* vecs;        // [n_comp][C]
@@ -116,75 +118,139 @@ __device__ __forceinline__ float layer_val(const void* data, int dtype, int64_t 
   return ((const float*)data)[off];
 }
 
+// four consecutive values of a row, 16-byte (float32) or 8-byte (16-bit) aligned
+__device__ __forceinline__ float4 layer_val4(const void* data, int dtype, int64_t off) {
+  if (dtype == MEM_F32) return *reinterpret_cast<const float4*>((const float*)data + off);
+  const uint2 q = *reinterpret_cast<const uint2*>((const uint16_t*)data + off);
+  const float2 a = dtype == MEM_BF16 ? __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.x))
+                                     : __half22float2(*reinterpret_cast<const __half2*>(&q.x));
+  const float2 b = dtype == MEM_BF16 ? __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.y))
+                                     : __half22float2(*reinterpret_cast<const __half2*>(&q.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+
 // the fixed cell range of block b of `blocks` over W2 cells
 __device__ __forceinline__ void block_range(u32 W2, int b, int blocks, u32& c0, u32& c1) {
   c0 = (u32)(((uint64_t)W2 * b) / blocks);
   c1 = (u32)(((uint64_t)W2 * (b + 1)) / blocks);
 }
 
+// A warp takes 32 cells' flags at a time and adds the observed rows, kMeanU of them
+// in flight, its lanes over the channels (lane, lane + 32, ...): whole lines, where a
+// thread per (cell, channel) with four cells in flight was bound by its chain of
+// loads (64 float32 channels of 500 x 500 cells: 63 -> 16 us).
+constexpr int kMeanU = 8;
+
 __global__ void __launch_bounds__(256) k_pca_mean(MapDev md, PcaArgs a) {
-  // thread t: column c = t % (C + 1) (column C counts the cells), cell lane t / (C + 1);
-  // lanes take every lanes-th cell of the block's range, four at a time
-  __shared__ float part[256];
+  constexpr int T = kPcaMaxC / 32;
+  __shared__ float part[8][kPcaMaxC + 1];
   u32 c0, c1;
   block_range(md.W2, blockIdx.x, a.blocks, c0, c1);
   const u32 base = (u32)a.map * md.W2;
-  const int cols = a.C + 1, lanes = blockDim.x / cols;
-  const int c = threadIdx.x % cols, lane = threadIdx.x / cols;
-  float s = 0.f;
-  if (lane < lanes) {
-    float q[4] = {0.f, 0.f, 0.f, 0.f};
-    for (u32 p = c0 + lane; p < c1; p += 4 * lanes) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float sum[T];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const u32 pu = p + u * lanes;
-        if (pu < c1 && (md.flags[base + pu] & a.obs_bit))
-          q[u] += c < a.C ? layer_val(a.data, a.dtype, (int64_t)(base + pu) * a.S + c) : 1.f;
+  for (int t = 0; t < T; ++t) sum[t] = 0.f;
+  u32 cnt = 0;
+  for (u32 p0 = c0 + warp * 32; p0 < c1; p0 += 256) {
+    u32 m = __ballot_sync(0xffffffffu, p0 + lane < c1 && (md.flags[base + p0 + lane] & a.obs_bit));
+    cnt += __popc(m);
+    while (m) {
+      float v[kMeanU][T];
+#pragma unroll
+      for (int u = 0; u < kMeanU; ++u) {
+        const int r = __ffs(m) - 1;  // -1 when none is left
+        m &= m - 1;
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+          const int c = lane + 32 * t;
+          v[u][t] = (r >= 0 && c < a.C) ? layer_val(a.data, a.dtype, (int64_t)(base + p0 + r) * a.S + c) : 0.f;
+        }
       }
+#pragma unroll
+      for (int u = 0; u < kMeanU; ++u)
+#pragma unroll
+        for (int t = 0; t < T; ++t) sum[t] += v[u][t];
     }
-    s = (q[0] + q[1]) + (q[2] + q[3]);
   }
-  part[threadIdx.x] = s;
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+    if (lane + 32 * t < a.C) part[warp][lane + 32 * t] = sum[t];
+  if (lane == 0) part[warp][a.C] = (float)cnt;  // below 2^24 for every block of a map of 2^28 cells
   __syncthreads();
-  if (threadIdx.x < cols) {
-    float t = 0.f;
-    for (int l = 0; l < lanes; ++l) t += part[l * cols + threadIdx.x];
-    a.mean_part[(int64_t)blockIdx.x * cols + threadIdx.x] = (double)t;
+  for (int c = threadIdx.x; c <= a.C; c += 256) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += (double)part[w][c];
+    a.mean_part[(int64_t)blockIdx.x * (a.C + 1) + c] = t;
   }
 }
 
-__global__ void k_pca_mean_final(PcaArgs a) {
-  for (int c = threadIdx.x; c <= a.C; c += blockDim.x) {
+// The blocks' sums in a fixed order: 1024 / 32 groups of blocks per column side by
+// side, then the groups (one thread per column walking every block took 135 us).
+__global__ void __launch_bounds__(1024) k_pca_mean_final(PcaArgs a) {
+  __shared__ double part[32][33];
+  __shared__ double tot[kPcaMaxC + 1];
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+  for (int cb = 0; cb <= a.C; cb += 32) {
+    const int c = cb + lane;
     double s = 0.0;
-    for (int b = 0; b < a.blocks; ++b) s += a.mean_part[(int64_t)b * (a.C + 1) + c];
-    a.mean_part[(int64_t)a.blocks * (a.C + 1) + c] = s;  // totals after the partials
+    if (c <= a.C)
+#pragma unroll 8
+      for (int b = grp; b < a.blocks; b += 32) s += a.mean_part[(int64_t)b * (a.C + 1) + c];
+    part[grp][lane] = s;
+    __syncthreads();
+    if (grp == 0 && c <= a.C) {
+      double t = 0.0;
+      for (int g = 0; g < 32; ++g) t += part[g][lane];
+      tot[c] = t;
+      a.mean_part[(int64_t)a.blocks * (a.C + 1) + c] = t;  // totals after the partials
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  const double n = a.mean_part[(int64_t)a.blocks * (a.C + 1) + a.C];
-  for (int c = threadIdx.x; c < a.C; c += blockDim.x)
-    a.mean[c] = n > 0.0 ? (float)(a.mean_part[(int64_t)a.blocks * (a.C + 1) + c] / n) : 0.f;
+  const double n = tot[a.C];
+  for (int c = threadIdx.x; c < a.C; c += blockDim.x) a.mean[c] = n > 0.0 ? (float)(tot[c] / n) : 0.f;
 }
 
-// partial covariance sums of one block's cells: thread (ty, tx) owns rows
-// ty*T .. and columns tx*T .. of the C x C matrix (T = ceil(C / 16))
-template <int T>
-__global__ void __launch_bounds__(256) k_pca_cov(MapDev md, PcaArgs a) {
-  __shared__ float xs[kPcaRows][kPcaMaxC + 1];
+// Partial covariance sums of one block's cells. The C x C matrix is cut into 8 x 8
+// tiles; the tiles on and above the diagonal, nt (nt + 1) / 2 with nt = ceil(C / 8),
+// are the matrix. A thread owns one of them for every `groups`-th staged row
+// (groups = the times the tiles fit 256 threads, at most 8): 64 FMAs for four
+// 16-byte reads of a row, half the products of the full matrix. FP32 FMAs bound it
+// (64 channels of 175k cells: 0.4 G FMAs); 100 -> 48 us against 4 x 4 tiles of the
+// full matrix fed by scalar reads. Rows are staged four channels per thread and load,
+// kCovU loads in flight (scalar staging loads took 111 us). A group's sums are added to the others' in group
+// order.
+constexpr int kCovU = 4;
+
+__global__ void __launch_bounds__(256) k_pca_cov(MapDev md, PcaArgs a, int nt, int tiles, int groups) {
+  extern __shared__ __align__(16) float xs[];  // [kPcaRows][ld], then reused for the groups' sums [tiles][64]
+  const int Cp = nt * 8, ld = Cp + 4;
+  __shared__ u32 wcnt[8];
+  __shared__ u32 list[256];
+  __shared__ __align__(16) float sm[kPcaMaxC];
+  if (threadIdx.x < a.C) sm[threadIdx.x] = a.mean[threadIdx.x];
+  for (int e = threadIdx.x; e < kPcaRows * ld; e += 256) xs[e] = 0.f;  // the columns past C stay 0
   u32 c0, c1;
   block_range(md.W2, blockIdx.x, a.blocks, c0, c1);
   const u32 base = (u32)a.map * md.W2;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float acc[T][T];
+  const int grp = threadIdx.x / tiles, tile = threadIdx.x - grp * tiles;
+  const bool on = grp < groups;
+  int ti = 0, tj = tile;  // row-major over the upper triangle
+  while (tj >= nt - ti) {
+    tj -= nt - ti;
+    ++ti;
+  }
+  tj += ti;
+  float acc[8][8];
 #pragma unroll
-  for (int i = 0; i < T; ++i)
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int k = 0; k < T; ++k) acc[i][k] = 0.f;
+    for (int k = 0; k < 8; ++k) acc[i][k] = 0.f;
   for (u32 p0 = c0; p0 < c1; p0 += 256) {
-    // list the observed cells of the next 256 (in cell order), then stage them 32 at a time
+    // list the observed cells of the next 256 (in cell order), then stage them kPcaRows at a time
     const u32 p = p0 + threadIdx.x;
-    const bool on = p < c1 && (md.flags[base + p] & a.obs_bit);
-    __shared__ u32 wcnt[8];
-    const u32 bal = __ballot_sync(0xffffffffu, on);
+    const bool obs = p < c1 && (md.flags[base + p] & a.obs_bit);
+    const u32 bal = __ballot_sync(0xffffffffu, obs);
     if ((threadIdx.x & 31) == 0) wcnt[threadIdx.x >> 5] = __popc(bal);
     __syncthreads();
     int before = 0, total = 0;
@@ -192,69 +258,146 @@ __global__ void __launch_bounds__(256) k_pca_cov(MapDev md, PcaArgs a) {
       before += w < (int)(threadIdx.x >> 5) ? (int)wcnt[w] : 0;
       total += (int)wcnt[w];
     }
-    const int my = before + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u));
-    __shared__ u32 list[256];
-    if (on) list[my] = p;
+    if (obs) list[before + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u))] = p;
     __syncthreads();
     for (int r0 = 0; r0 < total; r0 += kPcaRows) {
       const int nr = min(kPcaRows, total - r0);
-      for (int e = threadIdx.x; e < nr * a.C; e += blockDim.x) {
-        const int r = e / a.C, c = e - r * a.C;
-        xs[r][c] = __fsub_rn(layer_val(a.data, a.dtype, (int64_t)(base + list[r0 + r]) * a.S + c), a.mean[c]);
+      if ((a.C & 3) == 0) {  // rows (S = C values) then start on 16-byte (8-byte) boundaries
+        const int C4 = a.C >> 2;
+        for (int e0 = threadIdx.x; e0 < nr * C4; e0 += 256 * kCovU) {
+          float4 v[kCovU];
+#pragma unroll
+          for (int u = 0; u < kCovU; ++u) {
+            const int e = e0 + u * 256, r = e / C4;
+            if (e < nr * C4) v[u] = layer_val4(a.data, a.dtype, (int64_t)(base + list[r0 + r]) * a.S + 4 * (e - r * C4));
+          }
+#pragma unroll
+          for (int u = 0; u < kCovU; ++u) {
+            const int e = e0 + u * 256, r = e / C4, c = 4 * (e - r * C4);
+            if (e >= nr * C4) continue;
+            const float4 m = *reinterpret_cast<const float4*>(sm + c);
+            *reinterpret_cast<float4*>(xs + r * ld + c) = make_float4(
+                __fsub_rn(v[u].x, m.x), __fsub_rn(v[u].y, m.y), __fsub_rn(v[u].z, m.z), __fsub_rn(v[u].w, m.w));
+          }
+        }
+      } else {
+#pragma unroll 4
+        for (int e = threadIdx.x; e < nr * a.C; e += 256) {
+          const int r = e / a.C, c = e - r * a.C;
+          xs[r * ld + c] = __fsub_rn(layer_val(a.data, a.dtype, (int64_t)(base + list[r0 + r]) * a.S + c), sm[c]);
+        }
       }
       __syncthreads();
-      for (int r = 0; r < nr; ++r) {
-        float xa[T], xb[T];
+      if (on)
+        for (int r = grp; r < nr; r += groups) {
+          const float4* xa = reinterpret_cast<const float4*>(xs + r * ld + ti * 8);
+          const float4* xb = reinterpret_cast<const float4*>(xs + r * ld + tj * 8);
+          const float4 a0 = xa[0], a1 = xa[1], b0 = xb[0], b1 = xb[1];
+          const float va[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+          const float vb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-        for (int i = 0; i < T; ++i) {
-          const int ra = ty * T + i, cb = tx * T + i;
-          xa[i] = ra < a.C ? xs[r][ra] : 0.f;
-          xb[i] = cb < a.C ? xs[r][cb] : 0.f;
+          for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc[i][k] = __fmaf_rn(va[i], vb[k], acc[i][k]);
         }
-#pragma unroll
-        for (int i = 0; i < T; ++i)
-#pragma unroll
-          for (int k = 0; k < T; ++k) acc[i][k] = __fmaf_rn(xa[i], xb[k], acc[i][k]);
-      }
       __syncthreads();
     }
   }
-  float* out = a.cov_part + (int64_t)blockIdx.x * a.C * a.C;
+  for (int g = 0; g < groups; ++g) {  // the groups' sums in group order
+    if (on && grp == g) {
 #pragma unroll
-  for (int i = 0; i < T; ++i)
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int k = 0; k < T; ++k) {
-      const int ra = ty * T + i, cb = tx * T + k;
-      if (ra < a.C && cb < a.C) out[ra * a.C + cb] = acc[i][k];
+        for (int k = 0; k < 8; ++k) {
+          float* d = xs + (i * 8 + k) * tiles + tile;  // consecutive threads, consecutive words
+          *d = g ? *d + acc[i][k] : acc[i][k];
+        }
     }
+    __syncthreads();
+  }
+  float* out = a.cov_part + (int64_t)blockIdx.x * tiles * 64;
+  for (int e = threadIdx.x; e < tiles * 64; e += 256) out[e] = xs[e];
 }
 
-__global__ void k_pca_cov_final(PcaArgs a) {
+// The partial matrices in a fixed order, in float64: 8 groups of blocks per element
+// side by side, then the groups (one thread per element walking every block: 106 -> 12 us).
+__global__ void __launch_bounds__(256) k_pca_cov_final(PcaArgs a, int nt, int tiles) {
+  __shared__ double part[8][33];
   const double n = a.mean_part[(int64_t)a.blocks * (a.C + 1) + a.C];
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < a.C * a.C; e += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < a.blocks; ++b) s += (double)a.cov_part[(int64_t)b * a.C * a.C + e];
-    a.cov[e] = n > 0.0 ? (float)(s / n) : 0.f;
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (e < tiles * 64)
+#pragma unroll 8
+    for (int b = grp; b < a.blocks; b += 8) s += (double)a.cov_part[(int64_t)b * tiles * 64 + e];
+  part[grp][lane] = s;
+  __syncthreads();
+  if (grp != 0 || e >= tiles * 64) return;
+  double t = 0.0;
+  for (int g = 0; g < 8; ++g) t += part[g][lane];
+  const float v = n > 0.0 ? (float)(t / n) : 0.f;
+  const int ik = e / tiles, tile = e - ik * tiles;
+  int ti = 0, tj = tile;
+  while (tj >= nt - ti) {
+    tj -= nt - ti;
+    ++ti;
+  }
+  tj += ti;
+  const int row = ti * 8 + ik / 8, col = tj * 8 + ik % 8;
+  if (row < a.C && col < a.C) {
+    a.cov[row * a.C + col] = v;
+    a.cov[col * a.C + row] = v;
   }
 }
 
 // Cyclic Jacobi with round-robin pairs on the C x C covariance (C padded to an
 // even n with a zero row and column), in shared memory; one block of 1024.
+// A step rotates n / 2 disjoint pairs: A <- J^T A J falls apart into the 2 x 2
+// blocks (pair, pair), so a thread applies both sides to its block at once; then
+// warp 0 finds the next step's angles while the others bring V up to date (two
+// barriers a step; the pairs of step t are computed from t; a warp per row of
+// blocks, so no divisions). Bound by the latency of its steps; with the sides one
+// after the other, V with them and the round-robin order moved along by one
+// thread (four barriers a step) 64 channels took 609 us, now 314 us.
+// the angles of step `step`: round-robin, position 0 holds row 0, position i >= 1 row
+// 1 + (i - 1 - step) mod (n - 1); pair m: positions m and n - 1 - m. By one warp.
+__device__ __forceinline__ void jacobi_angles(const float* A, int ld, int n, int step, float4* rot) {
+  for (int m = threadIdx.x & 31; m < n / 2; m += 32) {
+    int i1 = m - 1 - step, i2 = n - 2 - m - step;
+    if (i1 < 0) i1 += n - 1;
+    if (i2 < 0) i2 += n - 1;
+    int p = m == 0 ? 0 : 1 + i1, q = 1 + i2;
+    if (p > q) {
+      const int t = p;
+      p = q;
+      q = t;
+    }
+    const float apq = A[p * ld + q], app = A[p * ld + p], aqq = A[q * ld + q];
+    float c = 1.f, s = 0.f;
+    if (apq != 0.f) {
+      const float tau = (aqq - app) / (2.f * apq);
+      const float t = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
+      c = 1.f / sqrtf(1.f + t * t);
+      s = t * c;
+    }
+    rot[m] = make_float4(c, s, __int_as_float(p), __int_as_float(q));
+  }
+}
+
 __global__ void __launch_bounds__(1024) k_pca_eig(PcaArgs a) {
   extern __shared__ float sm[];
   const int C = a.C, n = (C + 1) & ~1;
   float* A = sm;                 // [n][n + 1]
   float* V = A + n * (n + 1);    // [n][n + 1]
-  float* cs = V + n * (n + 1);   // [n / 2][2] rotation cosines and sines
-  int* pr = (int*)(cs + n);      // [n] round-robin positions
+  float4* rot = reinterpret_cast<float4*>(((uintptr_t)(V + n * (n + 1)) + 15) & ~(uintptr_t)15);  // [2][n / 2] cosine, sine, rows p < q
   __shared__ float s_off, s_tot;
-  const int ld = n + 1;
+  const int ld = n + 1, h = n / 2;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     const int i = e / n, k = e - i * n;
     A[i * ld + k] = (i < C && k < C) ? a.cov[i * C + k] : 0.f;
     V[i * ld + k] = i == k ? 1.f : 0.f;
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) pr[i] = i;
   __syncthreads();
   __shared__ float red[2][32];
   // converged when the off-diagonal mass is at the float32 rounding level of the matrix
@@ -288,86 +431,89 @@ __global__ void __launch_bounds__(1024) k_pca_eig(PcaArgs a) {
     }
     __syncthreads();
     if (!(s_off > conv * s_tot)) break;
+    if (warp == 0) jacobi_angles(A, ld, n, 0, rot);
+    __syncthreads();
     for (int step = 0; step < n - 1; ++step) {
-      // pair m: positions m and n - 1 - m of the round-robin order
-      for (int m = threadIdx.x; m < n / 2; m += blockDim.x) {
-        int p = pr[m], q = pr[n - 1 - m];
-        if (p > q) {
-          const int t = p;
-          p = q;
-          q = t;
+      const float4* ro = rot + (step & 1) * h;
+      for (int m1 = warp; m1 < h; m1 += 32) {  // A: rows of pair m1 first, then columns of pair m2
+        const float4 r1 = ro[m1];
+        float* rp = A + __float_as_int(r1.z) * ld;
+        float* rq = A + __float_as_int(r1.w) * ld;
+        for (int m2 = lane; m2 < h; m2 += 32) {
+          const float4 r2 = ro[m2];
+          const int p2 = __float_as_int(r2.z), q2 = __float_as_int(r2.w);
+          const float app = rp[p2], apq = rp[q2], aqp = rq[p2], aqq = rq[q2];
+          const float bpp = r1.x * app - r1.y * aqp, bqp = r1.y * app + r1.x * aqp;
+          const float bpq = r1.x * apq - r1.y * aqq, bqq = r1.y * apq + r1.x * aqq;
+          rp[p2] = r2.x * bpp - r2.y * bpq;
+          rp[q2] = r2.y * bpp + r2.x * bpq;
+          rq[p2] = r2.x * bqp - r2.y * bqq;
+          rq[q2] = r2.y * bqp + r2.x * bqq;
         }
-        const float apq = A[p * ld + q], app = A[p * ld + p], aqq = A[q * ld + q];
-        float c = 1.f, s = 0.f;
-        if (apq != 0.f) {
-          const float tau = (aqq - app) / (2.f * apq);
-          const float t = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
-          c = 1.f / sqrtf(1.f + t * t);
-          s = t * c;
-        }
-        cs[2 * m] = c;
-        cs[2 * m + 1] = s;
       }
       __syncthreads();
-      // rows: A <- J^T A (pair m mixes rows p and q)
-      for (int e = threadIdx.x; e < (n / 2) * n; e += blockDim.x) {
-        const int m = e / n, k = e - m * n;
-        int p = pr[m], q = pr[n - 1 - m];
-        if (p > q) {
-          const int t = p;
-          p = q;
-          q = t;
+      if (warp == 0) {
+        if (step + 1 < n - 1) jacobi_angles(A, ld, n, step + 1, rot + ((step + 1) & 1) * h);
+      } else {
+        for (int m2 = lane; m2 < h; m2 += 32) {  // V <- V J
+          const float4 r2 = ro[m2];
+          const int p2 = __float_as_int(r2.z), q2 = __float_as_int(r2.w);
+          for (int k = warp - 1; k < n; k += 31) {
+            float* vr = V + k * ld;
+            const float vp = vr[p2], vq = vr[q2];
+            vr[p2] = r2.x * vp - r2.y * vq;
+            vr[q2] = r2.y * vp + r2.x * vq;
+          }
         }
-        const float c = cs[2 * m], s = cs[2 * m + 1];
-        const float ap = A[p * ld + k], aq = A[q * ld + k];
-        A[p * ld + k] = c * ap - s * aq;
-        A[q * ld + k] = s * ap + c * aq;
-      }
-      __syncthreads();
-      // columns: A <- A J, V <- V J
-      for (int e = threadIdx.x; e < (n / 2) * n; e += blockDim.x) {
-        const int m = e / n, k = e - m * n;
-        int p = pr[m], q = pr[n - 1 - m];
-        if (p > q) {
-          const int t = p;
-          p = q;
-          q = t;
-        }
-        const float c = cs[2 * m], s = cs[2 * m + 1];
-        const float ap = A[k * ld + p], aq = A[k * ld + q];
-        A[k * ld + p] = c * ap - s * aq;
-        A[k * ld + q] = s * ap + c * aq;
-        const float vp = V[k * ld + p], vq = V[k * ld + q];
-        V[k * ld + p] = c * vp - s * vq;
-        V[k * ld + q] = s * vp + c * vq;
-      }
-      __syncthreads();
-      // next round-robin order: position 0 fixed, the others rotate by one
-      if (threadIdx.x == 0) {
-        const int last = pr[n - 1];
-        for (int i = n - 1; i > 1; --i) pr[i] = pr[i - 1];
-        pr[1] = last;
       }
       __syncthreads();
     }
   }
-  // the n_comp largest eigenvalues (the smaller index first on ties), signed vectors
-  if (threadIdx.x == 0) {
-    int used[kPcaMaxComp];
+  // the n_comp largest eigenvalues (the smaller index first on ties), each vector signed by its
+  // largest-magnitude component (the smaller index first on ties), by one warp
+  if (warp == 0) {
+    u32 taken = 0;  // bit j: diagonal entry lane + 32 j is used
     for (int k = 0; k < a.n_comp; ++k) {
-      int best = -1;
-      for (int i = 0; i < C; ++i) {
-        bool taken = false;
-        for (int j = 0; j < k; ++j) taken |= used[j] == i;
-        if (!taken && (best < 0 || A[i * ld + i] > A[best * ld + best])) best = i;
+      float bv = -INFINITY;
+      int bi = n;
+      for (int j = 0; lane + 32 * j < C; ++j) {
+        const float v = A[(lane + 32 * j) * (ld + 1)];
+        if (!((taken >> j) & 1u) && (bi == n || v > bv)) {
+          bv = v;
+          bi = lane + 32 * j;
+        }
       }
-      used[k] = best;
-      int big = 0;
-      for (int r = 1; r < C; ++r)
-        if (fabsf(V[r * ld + best]) > fabsf(V[big * ld + best])) big = r;
-      const float sg = V[big * ld + best] < 0.f ? -1.f : 1.f;
-      a.vals[k] = A[best * ld + best];
-      for (int r = 0; r < C; ++r) a.vecs[k * C + r] = sg * V[r * ld + best];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (oi < n && (bi == n || ov > bv || (ov == bv && oi < bi))) {
+          bv = ov;
+          bi = oi;
+        }
+      }
+      if ((bi & 31) == lane) taken |= 1u << (bi >> 5);
+      float mv = -1.f;
+      int mi = n;
+      for (int r = lane; r < C; r += 32) {
+        const float v = fabsf(V[r * ld + bi]);
+        if (v > mv) {
+          mv = v;
+          mi = r;
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, mv, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
+        if (ov > mv || (ov == mv && oi < mi)) {
+          mv = ov;
+          mi = oi;
+        }
+      }
+      const float sg = mi < n && V[mi * ld + bi] < 0.f ? -1.f : 1.f;
+      if (lane == 0) a.vals[k] = bv;
+      for (int r = lane; r < C; r += 32) a.vecs[k * C + r] = sg * V[r * ld + bi];
     }
   }
   __syncthreads();
@@ -378,13 +524,19 @@ __global__ void __launch_bounds__(1024) k_pca_eig(PcaArgs a) {
   }
 }
 
+// Four lanes per cell, four channels per lane and load (one channel where the row length
+// is not a multiple of 4), added over the lanes at the end: a thread per cell walked its row
+// alone, one 4-byte load at a time (64 channels, 500 x 500 cells: 62 -> 21 us).
 __global__ void __launch_bounds__(256) k_pca_project(MapDev md, PcaArgs a, int rx, int ry) {
-  __shared__ float sv[kPcaMaxComp * kPcaMaxC], sm[kPcaMaxC];
-  for (int e = threadIdx.x; e < a.n_comp * a.C; e += blockDim.x) sv[e] = a.vecs[e];
+  __shared__ __align__(16) float sv[kPcaMaxComp][kPcaMaxC], sm[kPcaMaxC];
+  for (int e = threadIdx.x; e < a.n_comp * a.C; e += blockDim.x) sv[e / a.C][e % a.C] = a.vecs[e];
   for (int c = threadIdx.x; c < a.C; c += blockDim.x) sm[c] = a.mean[c];
   __syncthreads();
-  const int W = md.W;
-  for (u32 j = blockIdx.x * blockDim.x + threadIdx.x; j < md.W2; j += gridDim.x * blockDim.x) {
+  const int W = md.W, sub = threadIdx.x & 3;
+  const bool vec = (a.C & 3) == 0;  // rows (S = C values) then start on 16-byte (8-byte) boundaries
+  for (u32 j0 = (blockIdx.x * blockDim.x + threadIdx.x) / 4; j0 - (threadIdx.x & 31) / 4 < md.W2;
+       j0 += gridDim.x * blockDim.x / 4) {  // the same count for every lane of a warp
+    const u32 j = min(j0, md.W2 - 1);
     const int ix = (int)(j % (u32)W), iy = (int)(j / (u32)W);
     int px = ix + rx;
     if (px >= W) px -= W;
@@ -395,14 +547,38 @@ __global__ void __launch_bounds__(256) k_pca_project(MapDev md, PcaArgs a, int r
 #pragma unroll
     for (int k = 0; k < kPcaMaxComp; ++k) out[k] = 0.f;
     if (md.flags[g] & a.obs_bit) {
-      for (int c = 0; c < a.C; ++c) {
-        const float x = __fsub_rn(layer_val(a.data, a.dtype, (int64_t)g * a.S + c), sm[c]);
+      if (vec) {
+#pragma unroll 4
+        for (int c = 4 * sub; c < a.C; c += 16) {
+          const float4 v = layer_val4(a.data, a.dtype, (int64_t)g * a.S + c);
+          const float4 m = *reinterpret_cast<const float4*>(sm + c);
+          const float x[4] = {__fsub_rn(v.x, m.x), __fsub_rn(v.y, m.y), __fsub_rn(v.z, m.z), __fsub_rn(v.w, m.w)};
 #pragma unroll
-        for (int k = 0; k < kPcaMaxComp; ++k)
-          if (k < a.n_comp) out[k] = __fmaf_rn(x, sv[k * a.C + c], out[k]);
+          for (int k = 0; k < kPcaMaxComp; ++k)
+            if (k < a.n_comp) {
+              const float4 w = *reinterpret_cast<const float4*>(&sv[k][c]);
+              out[k] = __fmaf_rn(x[0], w.x, out[k]);
+              out[k] = __fmaf_rn(x[1], w.y, out[k]);
+              out[k] = __fmaf_rn(x[2], w.z, out[k]);
+              out[k] = __fmaf_rn(x[3], w.w, out[k]);
+            }
+        }
+      } else {
+        for (int c = sub; c < a.C; c += 4) {
+          const float x = __fsub_rn(layer_val(a.data, a.dtype, (int64_t)g * a.S + c), sm[c]);
+#pragma unroll
+          for (int k = 0; k < kPcaMaxComp; ++k)
+            if (k < a.n_comp) out[k] = __fmaf_rn(x, sv[k][c], out[k]);
+        }
       }
     }
-    for (int k = 0; k < a.n_comp; ++k) a.proj[(int64_t)j * a.n_comp + k] = out[k];
+#pragma unroll
+    for (int k = 0; k < kPcaMaxComp; ++k) {
+      if (k >= a.n_comp) break;
+      out[k] += __shfl_xor_sync(0xffffffffu, out[k], 1);
+      out[k] += __shfl_xor_sync(0xffffffffu, out[k], 2);
+      if (sub == (k & 3) && j0 < md.W2) a.proj[(int64_t)j * a.n_comp + k] = out[k];
+    }
   }
 }
 
@@ -424,8 +600,10 @@ cudaError_t launch_normals(Map* m, int map_index, float* out, uint8_t* ok, cudaS
 cudaError_t launch_pca(Map* m, int map_index, int layer, int n_comp, float* proj, float* info, cudaStream_t st) {
   const LayerDev& L = m->Lh[layer];
   const int C = L.C;
-  const int blocks = m->n_sm * 4;
-  const size_t need = sizeof(double) * (size_t)(blocks + 1) * (C + 1) + sizeof(float) * (size_t)blocks * C * C +
+  const int nt = (C + 7) / 8, tiles = nt * (nt + 1) / 2;  // 8 x 8 tiles of the upper triangle
+  const int groups = std::max(1, std::min(8, 256 / tiles));
+  const int blocks = m->n_sm * kPcaBlocks;
+  const size_t need = sizeof(double) * (size_t)(blocks + 1) * (C + 1) + sizeof(float) * (size_t)blocks * tiles * 64 +
                       sizeof(float) * ((size_t)C * C + C + (size_t)kPcaMaxComp * (C + 1)) + 1024;
   if (need > m->pca_cap) {
     cudaError_t e = cudaStreamSynchronize(st);
@@ -451,7 +629,7 @@ cudaError_t launch_pca(Map* m, int map_index, int layer, int n_comp, float* proj
   a.mean_part = (double*)p;
   p += sizeof(double) * (size_t)(blocks + 1) * (C + 1);
   a.cov_part = (float*)p;
-  p += sizeof(float) * (size_t)blocks * C * C;
+  p += sizeof(float) * (size_t)blocks * tiles * 64;
   a.cov = (float*)p;
   p += sizeof(float) * (size_t)C * C;
   a.mean = (float*)p;
@@ -462,24 +640,22 @@ cudaError_t launch_pca(Map* m, int map_index, int layer, int n_comp, float* proj
   a.proj = proj;
   a.info = info;
   k_pca_mean<<<blocks, 256, 0, st>>>(m->md, a);
-  k_pca_mean_final<<<1, 256, 0, st>>>(a);
-  const int T = (C + 15) / 16;
-  if (T <= 1) k_pca_cov<1><<<blocks, 256, 0, st>>>(m->md, a);
-  else if (T <= 2) k_pca_cov<2><<<blocks, 256, 0, st>>>(m->md, a);
-  else if (T <= 4) k_pca_cov<4><<<blocks, 256, 0, st>>>(m->md, a);
-  else k_pca_cov<8><<<blocks, 256, 0, st>>>(m->md, a);
-  k_pca_cov_final<<<(C * C + 255) / 256, 256, 0, st>>>(a);
+  k_pca_mean_final<<<1, 1024, 0, st>>>(a);
   const int n = (C + 1) & ~1;
-  const size_t esm = sizeof(float) * (2 * (size_t)n * (n + 1) + n) + sizeof(int) * n;
+  // a staged block of rows, reused for the tiles' sums
+  const size_t csm = sizeof(float) * std::max((size_t)kPcaRows * (nt * 8 + 4), (size_t)tiles * 64);
+  const size_t esm = sizeof(float) * (2 * (size_t)n * (n + 1) + 4 * n) + 32;
   static bool attr[128] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 128 && !attr[dev]) {
     cudaError_t e = cudaFuncSetAttribute(k_pca_eig, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(float) * (2 * 128 * 129 + 128) + sizeof(int) * 128));
+                                         (int)(sizeof(float) * (2 * 128 * 129 + 4 * 128) + 32));
     if (e != cudaSuccess) return e;
     attr[dev] = true;
   }
+  k_pca_cov<<<blocks, 256, csm, st>>>(m->md, a, nt, tiles, groups);
+  k_pca_cov_final<<<tiles * 2, 256, 0, st>>>(a, nt, tiles);
   k_pca_eig<<<1, 1024, esm, st>>>(a);
   k_pca_project<<<m->n_sm * 4, 256, 0, st>>>(m->md, a, m->ring[2 * map_index], m->ring[2 * map_index + 1]);
   return cudaGetLastError();
