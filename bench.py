@@ -320,8 +320,8 @@ def run_ours(args):
     per_launch_s = cand[dom] / 1e3 / launches.get(dom, K)
     peak, peak_kind = peaks()
     achieved = algo[dom] / per_launch_s / 1e9
-    # the fuse kernel of the call: per-cell sums in registers where its summed columns (4 height
-    # sums, every source's channels, an arg-max pair per class-max source) fit one round of 32
+    # the fuse kernel of the call: the warp kernel where its summed columns (4 height sums, every
+    # source's channels, an arg-max pair per class-max source) fit its plan, as 32 certainly do
     fuse_name = "k_fuse_warps" if m.get_tuning()["fuse_kernel"] == 0 and fuse_columns <= 32 else "k_fuse_tiles"
     ncu_name = {"fuse_tiles": fuse_name, "radix_sort": "k_onesweep", "key": "k_points_key"}[dom]
     traffic = ncu_traffic(ncu_name)

@@ -274,10 +274,10 @@ mem_status mem_inject_fault(mem_map *m, int32_t kind);
 /* Schedule of the point path (results equal within float32 summation order;
  * each schedule is deterministic): radix_bits in [8, 10] is the digit width
  * of the key sort (at most 4 passes); blocks_per_sm in [1, 32] sizes the
- * persistent grids; fuse_kernel 0 sums a call's per-cell quantities in
- * registers, one point per lane (when its summed columns, 4 height sums plus
- * every source's channels and arg-max pair, number at most 32), 1 always in
- * shared-memory column walks over 128-point tiles. Synchronises the device. */
+ * persistent grids; fuse_kernel 0 lets every warp of a 128-point tile sum and
+ * fuse its own 32 points (when the call's summed columns, 4 height sums plus
+ * every source's channels and arg-max pair, fit six rounds of 32 and its tables),
+ * 1 always takes block-wide column walks over the tile. Synchronises the device. */
 mem_status mem_set_tuning(mem_map *m, int32_t radix_bits, int32_t blocks_per_sm, int32_t fuse_kernel);
 /* out = {radix_bits, blocks_per_sm, radix passes, fuse_kernel} (host). */
 mem_status mem_get_tuning(const mem_map *m, int32_t out[4]);

@@ -2,6 +2,7 @@
 // composition on the host (float64), and the move / layer-copy kernels.
 #include <math.h>
 #include <stdarg.h>
+#include <stddef.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -533,8 +534,9 @@ extern "C" mem_status mem_create_map(const mem_map_config* cfg, mem_map** out) {
 #undef ALLOC
   e = alloc_scratch(m, cfg->max_points > 0 ? cfg->max_points : (1 << 20));
   if (e != cudaSuccess) return bail(e, "alloc scratch");
-  // job block: header + per-map calls + offsets
-  m->job_bytes = sizeof(PointJob) + sizeof(MapCall) * cfg->n_maps + sizeof(int64_t) * (cfg->n_maps + 1) + 64;
+  // job block: header + fuse plan + per-map calls + offsets
+  m->job_bytes = sizeof(PointJob) + sizeof(memk::FusePlan) + sizeof(MapCall) * cfg->n_maps +
+                 sizeof(int64_t) * (cfg->n_maps + 1) + 64;
   e = dalloc(m, &p, m->job_bytes, false);
   if (e != cudaSuccess) return bail(e, "alloc job");
   m->d_job = (char*)p;
@@ -674,6 +676,90 @@ static mem_status check_sources(const Map* m, int32_t n_sources, const mem_sourc
   return MEM_OK;
 }
 
+// The warp fuse kernel's plan (n_rounds 0 when the call exceeds its tables).
+static void build_plan(memk::FusePlan& p, const PointJob& job, const LayerDev* L) {
+  using memk::kFuseQ;
+  memset(&p, 0, sizeof(p));
+  int r = 0, col = 4, ns = 0, nt = 0;
+  for (int c = 0; c < 4; ++c) p.slot[c] = (unsigned short)c;
+  auto close = [&]() {  // the round is full (or the call ends)
+    p.ncol[r] = col;
+    p.seg0[r + 1] = ns;
+    p.rule0[r + 1] = nt;
+    ++r;
+    col = 0;
+  };
+  for (int q = 0; q < job.n_src; ++q) {
+    const SrcDev& s = job.src[q];
+    const int pair = s.has_classmax ? 2 : 0;
+    for (int ch = 0; ch < s.C;) {
+      int n = std::min(kFuseQ - col, s.C - ch);
+      if (ch + n == s.C && col + n + pair > kFuseQ) --n;  // the pair stays with the last channels
+      if (ch + n < s.C) n = n >= 8 ? n & ~7 : n & ~3;     // rounds split rows at aligned channels
+      if (n <= 0) {
+        close();
+        if (r >= memk::kPlanRounds) return;
+        continue;
+      }
+      if (ns >= memk::kPlanSegs) return;
+      memk::PlanSeg& g = p.seg[ns++];
+      g.data = s.data;
+      g.C = s.C;
+      g.ch0 = ch;
+      g.n = n;
+      g.col = col;
+      g.dtype = s.dtype;
+      g.topk = s.topk;
+      g.vec = s.vec_ok && (s.C & 3) == 0;  // ch0 is a multiple of 4 wherever a row is split
+      const bool last = ch + n == s.C;
+      g.cm = s.has_classmax ? (last ? 2 : 1) : 0;
+      for (int k = 0; k < n + (last ? pair : 0); ++k) p.slot[r * kFuseQ + col + k] = (unsigned short)(s.acc_off + ch + k);
+      for (int b = 0; b < s.n_layers; ++b) {
+        const LayerDev& l = L[s.layers[b]];
+        const bool cm = l.rule == MEM_RULE_CLASSMAX;
+        if (cm && !last) continue;
+        if (nt >= memk::kPlanRules) return;
+        memk::PlanRule& t = p.rule[nt++];
+        t.data = l.data;
+        t.gvar = l.gvar;
+        t.w = l.w;
+        t.omw = l.one_minus_w;
+        t.var_meas = l.var_meas;
+        t.alpha0 = l.alpha0;
+        t.S = l.S;
+        t.ch = cm ? 0 : ch;
+        t.bit = 2u << s.layers[b];
+        t.col = cm ? col + n : col;
+        t.rule = l.rule;
+        t.dtype = l.dtype;
+        // 16-byte (float32: 4 values, 16-bit: 8) or 8-byte accesses where rows and groups are aligned to them
+        const int al = l.S | t.ch | n;
+        t.gw = cm ? 1 : (l.dtype != MEM_F32 && (al & 7) == 0) ? 8 : (al & 3) == 0 ? 4 : 1;
+        t.ng = cm ? 1 : n / t.gw;
+        t.inv = ((1u << 20) + (u32)t.ng - 1) / (u32)t.ng;
+      }
+      if (last && pair) p.am[r] |= 1u << (col + n);
+      col += n + (last ? pair : 0);
+      ch += n;
+    }
+    for (int b = 0; b < s.n_layers; ++b) {
+      const LayerDev& l = L[s.layers[b]];
+      p.all_bits |= 2u << s.layers[b];
+      if (l.rule == MEM_RULE_EXPAVG || l.rule == MEM_RULE_GAUSS || l.rule == MEM_RULE_DIRICHLET) {
+        p.row[p.n_rows].data = (const char*)l.data;
+        p.row[p.n_rows++].bytes = (int)dtype_size(l.dtype) * l.S;
+      }
+      if (l.rule == MEM_RULE_GAUSS) {
+        p.gauss[p.n_gauss].gvar = l.gvar;
+        p.gauss[p.n_gauss].var_meas = l.var_meas;
+        p.gauss[p.n_gauss++].bit = 2u << s.layers[b];
+      }
+    }
+  }
+  close();
+  p.n_rounds = r;
+}
+
 void memh::build_fuse_tables(PointJob& job, int acc_raw, const mem_map_config& cfg) {
   memk::FuseTables& f = job.ft;
   memset(&f, 0, sizeof(f));
@@ -765,8 +851,12 @@ static mem_status run_points(Map* m, int nm, const int64_t* offsets, int64_t n, 
   std::string buf(m->job_bytes, '\0');
   char* h = &buf[0];
   PointJob* job = (PointJob*)h;
-  MapCall* mcs = (MapCall*)(h + sizeof(PointJob));
-  int64_t* offs = (int64_t*)(h + sizeof(PointJob) + sizeof(MapCall) * nm);
+  // [job][plan][map calls][offsets]
+  constexpr size_t plan_at = (sizeof(PointJob) + 15) & ~(size_t)15, maps_at = plan_at + sizeof(memk::FusePlan);
+  memk::FusePlan* plan = (memk::FusePlan*)(h + plan_at);
+  MapCall* mcs = (MapCall*)(h + maps_at);
+  const size_t offs_at = (maps_at + sizeof(MapCall) * nm + 7) & ~(size_t)7;
+  int64_t* offs = (int64_t*)(h + offs_at);
   job->n = n;
   if (++m->call_id == 0) m->call_id = 1;  // 0 marks "never stamped"
   job->call_id = m->call_id;
@@ -780,7 +870,10 @@ static mem_status run_points(Map* m, int nm, const int64_t* offsets, int64_t n, 
     acc += src[q].C + 2 * src[q].has_classmax;  // channel sums, then (max value, class)
   }
   build_fuse_tables(*job, acc, m->cfg);
-  m->fuse_variant = job->ft.one_round ? 2 : 0;
+  build_plan(*plan, *job, m->Lh);
+  job->plan = (const memk::FusePlan*)(m->d_job + plan_at);
+  job->plan_vecs = (int)((offsetof(memk::FusePlan, rule) + sizeof(memk::PlanRule) * plan->rule0[plan->n_rounds]) / 16);
+  m->fuse_variant = plan->n_rounds == 0 ? 0 : (plan->n_rounds == 1 ? 2 : 6);
   for (int q = 0; q < n_src; ++q) m->fuse_variant |= src[q].topk ? 1 : 0;
   if (m->graph && m->graph_variant != m->fuse_variant) {  // the graph launches another kernel variant
     cudaGraphExecDestroy(m->graph);
@@ -793,18 +886,18 @@ static mem_status run_points(Map* m, int nm, const int64_t* offsets, int64_t n, 
     if (e != cudaSuccess) return cuda_fail(e, "partial-record buffer");
   }
   if (((uintptr_t)m->md.partial & 15) != 0) return fail(MEM_ERR_STATE, "fuse scratch not 16-byte aligned");
-  job->maps = (const MapCall*)(m->d_job + sizeof(PointJob));
-  job->offsets = nm > 1 ? (const int64_t*)(m->d_job + sizeof(PointJob) + sizeof(MapCall) * nm) : nullptr;
+  job->maps = (const MapCall*)(m->d_job + maps_at);
+  job->offsets = nm > 1 ? (const int64_t*)(m->d_job + offs_at) : nullptr;
   for (int b = 0; b < nm; ++b) {
     memset(&mcs[b], 0, sizeof(MapCall));
     pose_rel(T + 16 * b, &m->origin[2 * b], mcs[b]);
     mcs[b].ring_x = m->ring[2 * b];
     mcs[b].ring_y = m->ring[2 * b + 1];
   }
-  size_t bytes = sizeof(PointJob) + sizeof(MapCall) * nm;
+  size_t bytes = maps_at + sizeof(MapCall) * nm;
   if (nm > 1) {
     for (int b = 0; b <= nm; ++b) offs[b] = offsets[b];
-    bytes += sizeof(int64_t) * (nm + 1);
+    bytes = offs_at + sizeof(int64_t) * (nm + 1);
   }
   s = stage_job(m, h, bytes, ready ? job_st : st);
   if (s != MEM_OK) return s;

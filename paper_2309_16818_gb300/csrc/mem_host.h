@@ -25,7 +25,7 @@ struct Map {
   int key_bits = 1;
   uint32_t call_id = 0;  // point-path calls so far (the clean-up's per-cell stamps)
   // fuse kernel variant of the current point-path call: bit 0 a source has top-k rows,
-  // bit 1 its columns fit one round (the warp kernel runs instead of the tile kernel)
+  // bit 1 it fits the warp kernel's plan (else the tile kernel runs), bit 2 in several rounds
   int fuse_variant = 0;
   int graph_variant = -1;  // the variant the captured graph launches
   int n_sm = 148;

@@ -134,6 +134,55 @@ struct FuseTables {
   int any_gauss;
 };
 
+// The warp fuse kernel's plan of a call, built on the host: the call's columns (4
+// height sums, then per source its channels and, bound to a class-max layer, its
+// arg-max pair) cut into rounds of at most kFuseQ; per round the channels to stage
+// and the layers that take them. A call that does not
+// fit the plan's tables goes to the tile kernel.
+constexpr int kPlanRounds = 6;
+constexpr int kPlanSegs = 16;   // staged runs of a source's channels, all rounds
+constexpr int kPlanRules = 40;  // (layer, channels of a round), all rounds
+
+struct __align__(16) PlanSeg {
+  const void* data;
+  int C, ch0, n;       // row length, first channel, channels
+  int col;             // first stage column
+  int dtype;
+  int topk;            // > 0: rows of (class id, probability) pairs
+  int vec;             // 16-byte aligned data, C and ch0 multiples of 4
+  int cm;              // 1: the arg-max over the source's channels is tracked, 2: and ends here (pair at col + n)
+};
+
+// One layer over the channels that a round has of it, in groups of `gw` channels
+struct __align__(16) PlanRule {
+  void* data;          // layer values [cells][S]
+  float* gvar;         // GAUSS
+  float w, omw, var_meas, alpha0;
+  int S, ch;           // values per cell, first of the round's
+  u32 bit;             // the layer's observed bit
+  int col;             // first stage column
+  int rule, dtype;
+  int gw;              // channels per group: 8 (16-bit storage), 4 (rows of aligned groups), else 1
+  int ng;              // groups
+  u32 inv;             // ceil(2^20 / ng): k / ng = k * inv >> 20 for k < 32 ng, ng <= 32
+  int pad[3];
+};
+
+struct FusePlan {
+  int n_rounds;  // 0: the call does not fit the tables
+  u32 all_bits;  // observed bits of every layer of the call
+  int n_rows, n_gauss;
+  int seg0[kPlanRounds + 1], rule0[kPlanRounds + 1], ncol[kPlanRounds];
+  u32 am[kPlanRounds];     // arg-max value columns of the round
+  int pad[3];
+  unsigned short slot[kPlanRounds * kFuseQ];  // column -> word of a fuse slot
+  struct { const char* data; int bytes; int pad; } row[kMaxLayers];  // layer rows that a rule reads
+  struct { float* gvar; float var_meas; u32 bit; } gauss[kMaxLayers];
+  PlanSeg seg[kPlanSegs];
+  PlanRule rule[kPlanRules];  // last: the kernel copies the plan up to the rules in use
+};
+static_assert(sizeof(FusePlan) % 16 == 0 && sizeof(PlanRule) % 16 == 0, "copied in 16-byte words");
+
 // Per-call job of the point path, resident in device memory so the whole
 // kernel sequence can be replayed from a CUDA graph.
 struct PointJob {
@@ -147,6 +196,9 @@ struct PointJob {
   int acc;  // words per fuse slot: kSlotHdr, then per source C sums (+ max value, class)
   SrcDev src[kMaxSources];
   FuseTables ft;
+  const FusePlan* plan;  // 16-byte aligned; nullptr: no sources (one round of the 4 height sums)
+  int plan_vecs;         // its 16-byte words in use
+  int unused;
 };
 
 // ---------------------------------------------------------------------------

@@ -6,10 +6,11 @@
 //   k_onesweep      stable LSD radix-sort pass with decoupled look-back,
 //                   one per digit (keys = map * W*W + physical cell); each
 //                   CTA first scans the digit counts into global offsets
-//   k_fuse_tiles    per tile of sorted points: outlier gate, sums of every
+//   k_fuse_warps    per tile of sorted points: outlier gate, sums of every
 //                   cell's quantities (a reduce-by-key in a fixed order), then
 //                   for the cells inside the tile the Kalman height update and
-//                   every multi-modal layer's rule
+//                   every multi-modal layer's rule (k_fuse_tiles: the same for
+//                   calls of more columns than its plan holds)
 //   k_fuse_cross    the same for the cells whose points cross tiles (no float
 //                   atomics, fixed summation order: run-to-run identical)
 //
@@ -458,6 +459,8 @@ constexpr int kSegMax = 32;     // segments of a tile per walk
 constexpr int kStageU = 6;      // staging chunks in flight per thread
 constexpr int kStageV = 5;      // float4 row loads in flight per thread (warp fuse kernel)
 constexpr int kApplyU = 4;      // rule tasks in flight per thread
+constexpr int kWarpBlocks = 6;  // resident CTAs per SM of the warp fuse kernel (80 registers; 7: 48.6, 8: 48.1 us
+                                // against 43.4, from spills)
 constexpr int kCrossU = 8;      // slot pieces in flight per lane (runs crossing tiles)
 constexpr u32 kBitHead = 1u;    // slot bits: the run begins in the tile
 constexpr u32 kBitEnd = 2u;     //            the run ends in the tile
@@ -1324,85 +1327,173 @@ __device__ __forceinline__ void cross_run(const MapDev& md, const LayerDev* sL, 
 }
 
 // ---------------------------------------------------------------------------
-// 4b. the same fusion for calls whose columns fit one round (at most kQ), with
-//     the per-cell sums taken in registers. A warp holds 32 consecutive points
-//     of the tile, one per lane: each lane stages its point's channels in its
-//     own shared-memory row and adds the height sums after the gate; then every
-//     column is summed over the pieces of runs in the warp by a segmented
-//     inclusive scan of shuffles (the piece's sum lands on its last lane; an
-//     arg-max pair takes the segmented maximum instead). The lane where a run
-//     ends adds the pieces of the earlier warps of the tile that the run covers
-//     (in warp order) and fuses the run itself: every layer's rule over its
-//     cell's rows, class max, Kalman height update, Gaussian variances, flags.
-//     Runs that cross the tile's boundaries leave their sums and header in the
-//     tile's two slots exactly as k_fuse_tiles does, for k_fuse_cross.
+// 4b. the same fusion with the per-cell sums taken by warps, for calls that fit a
+//     FusePlan (up to 192 summed columns in rounds of 32; wider calls go to
+//     k_fuse_tiles). A warp holds 32 consecutive points of the tile, one per lane.
+//     Per round: each lane stages its point's channels in its own shared-memory row
+//     (round 0 adds the height sums after the gate); lane c walks column c down the
+//     warp's rows and leaves each piece's sum in the piece's last row (an arg-max
+//     pair takes the segmented maximum by shuffles); a run that began in an earlier
+//     warp of the tile gets the earlier pieces added, in warp order, by the lanes of
+//     the warp it ends in, one column each; then the runs that lie in the tile are
+//     fused by the warp they end in: layer by layer, a (run, group of channels) pair
+//     per lane, and in round 0 the Kalman height update by the lane where the run
+//     ends. Runs that cross the tile's boundaries leave their sums and header in
+//     the tile's two slots exactly as k_fuse_tiles does, for k_fuse_cross.
+//
+//     Bound by issue and by the latency of a tile's chain (keys -> state and rows ->
+//     sums -> layer rows). With one lane per run applying every layer (the lanes
+//     without a run end idle) and one lane adding the earlier warps' columns, the run
+//     ends took a quarter of the instructions and 40 % of the time. ncu, cold caches:
+//     447k kept points in 31k cells, 29 columns 59.4 -> 43.4 us (25.0 -> 20.4 M warp
+//     instructions); 288k points of 91 columns 243 (k_fuse_tiles) -> 87 us; 64 maps, 1.4
+//     points per cell 141 -> 132 us; 20k points 13.1 -> 10.2 us. One task list over all
+//     layers of a run (rules mixed in a warp) took 52 / 113 / 162 / 10.3 us.
 
-struct WarpSmem {
-  float stage[kFT * kQS];  // one row per point of the tile
-  SrcDev src[kMaxSources];
-  LayerDev L[kMaxLayers];
-  ChunkDesc ck[kQ];
-  MapCall mc0;
-  int rlay[kMaxSources][kMaxSrcLayers];  // per source: its layers other than class max
-  int nrlay[kMaxSources];
-  int qc0[kMaxSources], qch0[kMaxSources], qn[kMaxSources];
-  int pair_col[kMaxSources];
-  int n_ck, n_pair;
-  u32 whd[kFT / 32];  // per warp: the lanes where a run begins
+struct FwRun {
+  u32 g, fl;  // cell, pre-call flags
+  float n;    // points
+  int row;    // stage row of the sums
 };
 
-// One rule layer over the channels of a run, by the lane that fuses it: old
-// values (and the Gaussian prior variance) first, kRuleU vectors in flight.
-template <int RULE, int DT, int W>
-__device__ __forceinline__ void lane_rule_t(const LayerDev& L, int l, const float* S, int ch0, int nch, u32 g,
-                                            u32 fl, float N, float rN) {
-  constexpr int kRuleU = 5;
-  const bool obs = (fl & (2u << l)) != 0;
-  const float s02 = (RULE == MEM_RULE_GAUSS && obs) ? L.gvar[g] : 0.f;
-  const RuleCoef co = rule_coef(L, N, rN, obs, s02);
-  const int64_t base = (int64_t)g * L.S + ch0;
-  for (int k0 = 0; k0 < nch; k0 += kRuleU * W) {
-    float old[kRuleU][W];
+struct __align__(16) WarpSmem {
+  float stage[kFT * kQS];  // one row per point of the tile
+  FusePlan plan;
+  FwRun run[kFT / 32][32];  // per warp: the runs that it fuses
+  MapCall mc0;
+  u32 whd[kFT / 32];  // per warp: the lanes where a run begins
+};
+static_assert(sizeof(FwRun) == 16, "read as one word");
+
+// GW consecutive values of a layer row (GW == 1: any offset)
+template <int GW>
+__device__ __forceinline__ void ld_group(const PlanRule& t, int64_t off, float o[GW]) {
+  if (GW == 1) {
+    o[0] = t.dtype == MEM_F32    ? ld1t<MEM_F32>(t.data, off)
+           : t.dtype == MEM_BF16 ? ld1t<MEM_BF16>(t.data, off)
+                                 : ld1t<MEM_F16>(t.data, off);
+  } else if (GW == 4) {
+    if (t.dtype == MEM_F32) ld4t<MEM_F32>(t.data, off, o);
+    else if (t.dtype == MEM_BF16) ld4t<MEM_BF16>(t.data, off, o);
+    else ld4t<MEM_F16>(t.data, off, o);
+  } else {  // 16-bit storage
+    const uint4 q = *reinterpret_cast<const uint4*>((const uint16_t*)t.data + off);
+    const u32 w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-    for (int u = 0; u < kRuleU; ++u) {
-      const int k = k0 + u * W;
+    for (int k = 0; k < 4; ++k) {
+      const float2 f = t.dtype == MEM_BF16 ? __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[k]))
+                                           : __half22float2(*reinterpret_cast<const __half2*>(&w[k]));
+      o[2 * k] = f.x;
+      o[2 * k + 1] = f.y;
+    }
+  }
+}
+template <int GW>
+__device__ __forceinline__ void st_group(const PlanRule& t, int64_t off, const float n[GW]) {
+  if (GW == 1) {
+    if (t.dtype == MEM_F32) st1t<MEM_F32>(t.data, off, n[0]);
+    else if (t.dtype == MEM_BF16) st1t<MEM_BF16>(t.data, off, n[0]);
+    else st1t<MEM_F16>(t.data, off, n[0]);
+  } else if (GW == 4) {
+    if (t.dtype == MEM_F32) st4t<MEM_F32>(t.data, off, n);
+    else if (t.dtype == MEM_BF16) st4t<MEM_BF16>(t.data, off, n);
+    else st4t<MEM_F16>(t.data, off, n);
+  } else {
+    u32 w[4];
 #pragma unroll
-      for (int w = 0; w < W; ++w) old[u][w] = 0.f;
-      if (RULE != MEM_RULE_LATEST && obs && k < nch) {
-        if (W == 4) ld4t<DT>(L.data, base + k, old[u]);
-        else old[u][0] = ld1t<DT>(L.data, base + k);
+    for (int k = 0; k < 4; ++k) {
+      if (t.dtype == MEM_BF16) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(n[2 * k], n[2 * k + 1]);
+        w[k] = *reinterpret_cast<const u32*>(&a);
+      } else {
+        const __half2 a = __floats2half2_rn(n[2 * k], n[2 * k + 1]);
+        w[k] = *reinterpret_cast<const u32*>(&a);
+      }
+    }
+    *reinterpret_cast<uint4*>((uint16_t*)t.data + off) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// One layer over the warp's nrun runs: a lane takes a (run, group) pair, two of
+// them (one of eight values) with their old values (and Gaussian prior variances) in flight. The layer is
+// the warp's, so its rule and storage cost no divergence; every rule is
+//   new = c1 old + c2 (m S):  LATEST 0, 1, 1/N;  EXPAVG 1 - w, w, 1/N;  DIRICHLET
+//   1, 1, 1 (old = alpha0 when unobserved);  GAUSS sf2/(N s02 + sf2),
+//   s02/(N s02 + sf2), 1;  and 0, 1, 1/N for the first observation of EXPAVG and GAUSS.
+template <int GW>
+__device__ __forceinline__ void run_rule(const WarpSmem& s, const PlanRule& t, const FwRun* runs, int nrun) {
+  constexpr int kTaskU = GW == 8 ? 1 : 2;
+  const int ng = t.ng, total = nrun * ng, rule = t.rule;
+  const u32 inv = t.inv, bit = t.bit;
+  for (int k0 = threadIdx.x & 31; k0 < total; k0 += 32 * kTaskU) {
+    float old[kTaskU][GW], s02[kTaskU];
+#pragma unroll
+    for (int u = 0; u < kTaskU; ++u) {
+      const int k = k0 + 32 * u;
+      s02[u] = 0.f;
+#pragma unroll
+      for (int w = 0; w < GW; ++w) old[u][w] = 0.f;
+      if (k >= total) continue;
+      const int i = (int)(((u32)k * inv) >> 20);  // k / ng
+      const u32 g = runs[i].g;
+      if (runs[i].fl & bit) {
+        if (rule != MEM_RULE_LATEST) ld_group<GW>(t, (int64_t)g * t.S + t.ch + (k - i * ng) * GW, old[u]);
+        if (rule == MEM_RULE_GAUSS) s02[u] = t.gvar[g];
+      } else if (rule == MEM_RULE_DIRICHLET) {
+#pragma unroll
+        for (int w = 0; w < GW; ++w) old[u][w] = t.alpha0;
       }
     }
 #pragma unroll
-    for (int u = 0; u < kRuleU; ++u) {
-      const int k = k0 + u * W;
-      if (k < nch) {
-        float nv[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) nv[w] = rule_value_t<RULE>(L, old[u][w], S[k + w], co);
-        if (W == 4) st4t<DT>(L.data, base + k, nv);
-        else st1t<DT>(L.data, base + k, nv[0]);
+    for (int u = 0; u < kTaskU; ++u) {
+      const int k = k0 + 32 * u;
+      if (k >= total) continue;
+      const int i = (int)(((u32)k * inv) >> 20), j = (k - i * ng) * GW;
+      const FwRun r = runs[i];
+      const bool obs = (r.fl & bit) != 0;
+      float c1 = 0.f, c2 = 1.f, m = 1.f;
+      if (rule == MEM_RULE_DIRICHLET) {
+        c1 = 1.f;
+      } else if (rule == MEM_RULE_GAUSS && obs) {
+        const float rden = __frcp_rn(__fmaf_rn(r.n, s02[u], t.var_meas));
+        c1 = t.var_meas * rden;
+        c2 = s02[u] * rden;
+      } else {
+        m = __frcp_rn(r.n);
+        if (rule == MEM_RULE_EXPAVG && obs) {
+          c1 = t.omw;
+          c2 = t.w;
+        }
       }
+      const float* S = s.stage + r.row * kQS + t.col + j;
+      float nv[GW];
+#pragma unroll
+      for (int w = 0; w < GW; ++w) nv[w] = fmaf(c1, old[u][w], c2 * (m * S[w]));
+      st_group<GW>(t, (int64_t)r.g * t.S + t.ch + j, nv);
     }
   }
 }
 
-__device__ __forceinline__ void lane_rule(const LayerDev& L, int l, const float* S, int ch0, int nch, u32 g, u32 fl,
-                                          float N, float rN) {
-  const bool v4 = (L.S & 3) == 0 && (ch0 & 3) == 0 && (nch & 3) == 0;
-#define MEM_LR(R, D)                                                \
-  case R * 4 + D:                                                   \
-    if (v4) lane_rule_t<R, D, 4>(L, l, S, ch0, nch, g, fl, N, rN);  \
-    else lane_rule_t<R, D, 1>(L, l, S, ch0, nch, g, fl, N, rN);     \
-    break;
-  switch (L.rule * 4 + L.dtype) {
-    MEM_LR(MEM_RULE_LATEST, MEM_F32) MEM_LR(MEM_RULE_LATEST, MEM_BF16) MEM_LR(MEM_RULE_LATEST, MEM_F16)
-    MEM_LR(MEM_RULE_EXPAVG, MEM_F32) MEM_LR(MEM_RULE_EXPAVG, MEM_BF16) MEM_LR(MEM_RULE_EXPAVG, MEM_F16)
-    MEM_LR(MEM_RULE_GAUSS, MEM_F32) MEM_LR(MEM_RULE_GAUSS, MEM_BF16) MEM_LR(MEM_RULE_GAUSS, MEM_F16)
-    MEM_LR(MEM_RULE_DIRICHLET, MEM_F32)
-    default: break;
+// the rules of a round over the warp's runs, layer by layer
+__device__ __forceinline__ void run_rules(const WarpSmem& s, const FwRun* runs, int nrun, int q0, int q1) {
+  for (int q = q0; q < q1; ++q) {
+    const PlanRule& t = s.plan.rule[q];
+    if (t.rule == MEM_RULE_CLASSMAX) {  // (value, class) of the arg-max pair, a lane per run
+      const int lane = threadIdx.x & 31;
+      if (lane < nrun) {
+        const FwRun& r = runs[lane];
+        const float* S = s.stage + r.row * kQS + t.col;
+        *reinterpret_cast<float2*>((float*)t.data + (int64_t)r.g * 2) =
+            make_float2(S[0] == -INFINITY ? -1.f : (float)__float_as_int(S[1]), S[0]);
+      }
+    } else if (t.gw == 4) {
+      run_rule<4>(s, t, runs, nrun);
+    } else if (t.gw == 8) {
+      run_rule<8>(s, t, runs, nrun);
+    } else {
+      run_rule<1>(s, t, runs, nrun);
+    }
   }
-#undef MEM_LR
 }
 
 // four (one) source values of any storage type, from their bits
@@ -1428,87 +1519,91 @@ __device__ __forceinline__ float ld1_any(const void* base, int dtype, int64_t of
   return dtype == MEM_BF16 ? __uint_as_float((u32)b << 16) : __half2float(__ushort_as_half(b));
 }
 
-// One source's channels of a point into its stage row (columns col0 .. col0 +
-// C - 1), then, for a source bound to a class-max layer, the point's largest
-// channel value and its channel (the smaller channel on ties) in the next two
-// columns. Rows of C % 4 == 0 channels of 16-byte aligned data are read four
+// A segment's channels of a point into its stage row. For a source bound to a
+// class-max layer the largest channel value so far and its channel (the smaller
+// channel on ties) go along in (pb, pi), and to the two columns after the source's
+// last channel. Rows of C % 4 == 0 channels of 16-byte aligned data are read four
 // channels at a time.
-__device__ __forceinline__ void stage_src(float* srow, const void* data, int dtype, int64_t id, int C, int col0,
-                                          bool vec, bool cm) {
-  float pb = -INFINITY;
-  int pi = 0x7fffffff;
-  const int64_t base = id * C;
-  if (vec && (C & 3) == 0) {
-    for (int k0 = 0; k0 < C; k0 += 4 * kStageV) {
+__device__ __forceinline__ void stage_seg(const PlanSeg& g, float* srow, int64_t id, float& pb, int& pi) {
+  const bool cm = g.cm != 0;
+  const int64_t base = id * g.C + g.ch0;
+  float* col = srow + g.col;
+  if (g.vec) {
+    for (int k0 = 0; k0 < g.n; k0 += 4 * kStageV) {
       float4 v[kStageV];
 #pragma unroll
       for (int u = 0; u < kStageV; ++u)
-        if (k0 + 4 * u < C) v[u] = ld4_any(data, dtype, base + k0 + 4 * u);
+        if (k0 + 4 * u < g.n) v[u] = ld4_any(g.data, g.dtype, base + k0 + 4 * u);
 #pragma unroll
       for (int u = 0; u < kStageV; ++u)
-        if (k0 + 4 * u < C)
+        if (k0 + 4 * u < g.n)
 #pragma unroll
           for (int w = 0; w < 4; ++w) {
             const float e = w == 0 ? v[u].x : w == 1 ? v[u].y : w == 2 ? v[u].z : v[u].w;
-            srow[col0 + k0 + 4 * u + w] = e;
+            col[k0 + 4 * u + w] = e;
             if (cm && e > pb) {
               pb = e;
-              pi = k0 + 4 * u + w;
+              pi = g.ch0 + k0 + 4 * u + w;
             }
           }
     }
   } else {
-    for (int k0 = 0; k0 < C; k0 += 8) {
+    for (int k0 = 0; k0 < g.n; k0 += 8) {
       float v[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (k0 + u < C) v[u] = ld1_any(data, dtype, base + k0 + u);
+        if (k0 + u < g.n) v[u] = ld1_any(g.data, g.dtype, base + k0 + u);
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (k0 + u < C) {
-          srow[col0 + k0 + u] = v[u];
+        if (k0 + u < g.n) {
+          col[k0 + u] = v[u];
           if (cm && v[u] > pb) {
             pb = v[u];
-            pi = k0 + u;
+            pi = g.ch0 + k0 + u;
           }
         }
     }
   }
-  if (cm) {
-    srow[col0 + C] = pb;
-    srow[col0 + C + 1] = __int_as_float(pi);
-  }
 }
 
-// The chunks of the top-k sources (rows of (class id, probability) pairs
-// expanded into channels), with their arg-max.
-__device__ __noinline__ void stage_topk_chunks(const ChunkDesc* ck, int nck, const SrcDev* src, float* srow,
-                                               int64_t id) {
-  float pb = -INFINITY;
-  int pi = 0x7fffffff;
-  for (int k = 0; k < nck; ++k) {
-    const ChunkDesc& d = ck[k];
-    if (!src[d.src].topk) continue;
-    float v[4];
-    ld_chunk<true>(d, id, v);
-    for (int w = 0; w < d.n; ++w) {
-      srow[d.col + w] = v[w];
-      if (d.am >= 0 && v[w] > pb) {
-        pb = v[w];
-        pi = d.ch0 + w;
+// The same for rows of (class id, probability) pairs: the segment's columns are
+// cleared, the listed probabilities added in row order, then the columns scanned.
+__device__ __noinline__ void stage_seg_topk(const PlanSeg& g, float* srow, int64_t id, float& pb, int& pi) {
+  const float* __restrict__ r = (const float*)g.data + id * 2 * g.topk;
+  float* col = srow + g.col;
+  for (int k = 0; k < g.n; ++k) col[k] = 0.f;
+  for (int j0 = 0; j0 < g.topk; j0 += 4) {
+    float ci[4], pr[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      ci[u] = -1.f;
+      if (j0 + u < g.topk) {
+        ci[u] = __ldg(r + 2 * (j0 + u));
+        pr[u] = __ldg(r + 2 * (j0 + u) + 1);
       }
     }
-    if (d.am >= 0 && (d.am >> 30)) {
-      srow[d.am & 0xffff] = pb;
-      srow[(d.am & 0xffff) + 1] = __int_as_float(pi);
-      pb = -INFINITY;
-      pi = 0x7fffffff;
-    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (ci[u] >= 0.f && ci[u] < (float)g.C && ci[u] == floorf(ci[u])) {
+        const int k = (int)ci[u] - g.ch0;
+        if (k >= 0 && k < g.n) col[k] = __fadd_rn(col[k], pr[u]);
+      }
   }
+  if (g.cm)
+    for (int k = 0; k < g.n; ++k) {
+      const float e = col[k];
+      if (e > pb) {
+        pb = e;
+        pi = g.ch0 + k;
+      }
+    }
 }
 
-template <bool TOPK, bool RAY>
-__global__ void __launch_bounds__(kFT, 6) k_fuse_warps(MapDev md, const PointJob* __restrict__ job, int sorted1) {
+// TOPK: some source has top-k rows; RAY: the map runs the ray-cast clean-up; MULTI:
+// the plan has several rounds (all known on the host)
+template <bool TOPK, bool RAY, bool MULTI>
+__global__ void __launch_bounds__(kFT, kWarpBlocks) k_fuse_warps(MapDev md, const PointJob* __restrict__ job,
+                                                                 int sorted1) {
   extern __shared__ __align__(16) unsigned char fw_raw[];
   WarpSmem& s = *reinterpret_cast<WarpSmem*>(fw_raw);
   if (*(volatile int*)md.err) return;  // a device error is pending: the point path does nothing
@@ -1516,40 +1611,33 @@ __global__ void __launch_bounds__(kFT, 6) k_fuse_warps(MapDev md, const PointJob
   const u32* __restrict__ sv = sorted1 ? md.vals1 : md.vals0;
   const int64_t n_kept = *(volatile u32*)&md.counters[6];
   const int n_tiles = (int)((n_kept + kFT - 1) / kFT);
-  const int n_src = job->n_src;
   const int acc = job->acc;
-  const FuseTables* __restrict__ ft = &job->ft;
-  const int G = ft->ncol;  // columns of the call (at most kQ)
-  const bool any_gauss = ft->any_gauss;
   const float* __restrict__ xyz = job->xyz;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const u64 call_hi = RAY ? (u64)job->call_id << 32 : 0ull;
-  // the call's tables (built on the host) into shared memory
-  if (t < n_src) s.src[t] = job->src[t];
-  if (t < md.n_layers) s.L[t] = md.L[t];
-  if (t < kQ) s.ck[t] = ft->ck[t];
-  if (t < kMaxSources) {
-    s.nrlay[t] = ft->nrlay[t];
-    for (int b = 0; b < kMaxSrcLayers; ++b) s.rlay[t][b] = ft->rlay[t][b];
-    s.qc0[t] = ft->qc0[t];
-    s.qch0[t] = ft->qch0[t];
-    s.qn[t] = ft->qn[t];
-    s.pair_col[t] = ft->pair_col[t];
+  if (blockIdx.x >= n_tiles) return;
+  // the call's plan (built on the host) into shared memory
+  if (job->plan) {
+    const uint4* ps = reinterpret_cast<const uint4*>(job->plan);
+    uint4* pd = reinterpret_cast<uint4*>(&s.plan);
+    const int nv = job->plan_vecs;
+    for (int i = t; i < nv; i += kFT) pd[i] = __ldg(ps + i);
+  } else {  // the height sums alone
+    if (t < 2) s.plan.seg0[t] = s.plan.rule0[t] = 0;
+    if (t < 4) s.plan.slot[t] = (unsigned short)t;
+    if (t == 0) {
+      s.plan.n_rounds = 1;
+      s.plan.all_bits = 0;
+      s.plan.n_rows = s.plan.n_gauss = 0;
+      s.plan.ncol[0] = 4;
+      s.plan.am[0] = 0;
+    }
   }
-  if (t == 0) {
-    s.mc0 = job->maps[0];
-    s.n_ck = ft->n_ck;
-    s.n_pair = ft->n_pair;
-  }
-  // columns of the arg-max pairs (value, channel): maxima, not sums
-  u32 am_val = 0;
-  for (int k = 0; k < ft->n_pair; ++k) am_val |= 1u << ft->pair_col[k];
-  const u32 am_any = am_val | (am_val << 1);
+  if (t == 0) s.mc0 = job->maps[0];
   const u32 le = 0xffffffffu >> (31 - lane);  // lanes up to this one
   u32 heads = 0;  // runs that begin at this thread's points
   float* srow = s.stage + t * kQS;
   for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    __syncthreads();  // tables in place; the previous tile is done with the stage
     const int64_t p0 = (int64_t)tile * kFT;
     const int np = (int)min((int64_t)kFT, n_kept - p0);
     const int64_t p = p0 + t;
@@ -1562,6 +1650,7 @@ __global__ void __launch_bounds__(kFT, 6) k_fuse_warps(MapDev md, const PointJob
       if (p > 0) kprev = sk[p - 1];
       if (p + 1 < n_kept) knext = sk[p + 1];
     }
+    __syncthreads();  // plan in place; the previous tile is done with the shared arrays
     const bool hd = on && key != kprev;  // a run begins here
     const bool ed = on && key != knext;  // a run ends here
     const bool tl = t == np - 1;         // the tile's last point
@@ -1585,171 +1674,204 @@ __global__ void __launch_bounds__(kFT, 6) k_fuse_warps(MapDev md, const PointJob
       ys = __ldg(xyz + 3 * (int64_t)id + 1);
       zs = __ldg(xyz + 3 * (int64_t)id + 2);
     }
-    if (ed) {  // rule layers' rows of a cell this lane may fuse, into L2
-      for (int q = 0; q < n_src; ++q)
-        for (int j = 0; j < s.nrlay[q]; ++j) {
-          const LayerDev& L = s.L[s.rlay[q][j]];
-          if (L.rule == MEM_RULE_LATEST) continue;
-          const int bytes = L.S * (L.dtype == MEM_F32 ? 4 : 2);
-          const char* row = (const char*)L.data + (int64_t)key * bytes;
-          for (int o = 0; o < bytes; o += 128) prefetch_l2(row + o);
-          prefetch_l2(row + bytes - 1);
-        }
-    }
-    // B. the point's channels into its row, with the arg-max of a class-max
-    //    source on the way (top-k sources by the chunk table)
-    if (on) {
-      for (int q = 0; q < n_src; ++q) {
-        const SrcDev& S = s.src[q];
-        if (TOPK && S.topk) continue;
-        stage_src(srow, S.data, S.dtype, id, S.C, s.qc0[q], S.vec_ok, S.has_classmax);
+    if (ed)  // rows that the rules of a cell fused here read, into L2
+      for (int k = 0; k < s.plan.n_rows; ++k) {
+        const int bytes = s.plan.row[k].bytes;
+        const char* row = s.plan.row[k].data + (int64_t)key * bytes;
+        for (int o = 0; o < bytes; o += 128) prefetch_l2(row + o);
+        prefetch_l2(row + bytes - 1);
       }
-      if (TOPK) stage_topk_chunks(s.ck, s.n_ck, s.src, srow, id);
-    }
-    // C. outlier gate against the pre-call state: the point's height sums
-    u64 zk = 0;  // ray-cast clean-up: (call id, lowest z) key of an accepted point
-    if (on) {
-      const MapCall* mc = md.n_maps > 1 ? job->maps + key / md.W2 : &s.mc0;
-      float z, vm;
-      eval_zvm(md, *mc, xs, ys, zs, z, vm);
-      const bool rej = (fl & kFlagValid) && gate_reject(z, h0, v0, vm, md.lam2);
-      const float w = __frcp_rn(vm);
-      srow[0] = rej ? 0.f : w;
-      srow[1] = rej ? 0.f : z * w;
-      srow[2] = rej ? 0.f : 1.f;
-      srow[3] = rej ? 1.f : 0.f;
-      if (RAY && !rej) zk = call_hi | (u64)(~ordered_bits(__float_as_uint(z)));
-    }
-    // D. sums over the pieces of runs in the warp: lane c walks column c down
-    //    the warp's rows in point order and leaves each piece's sum in the
-    //    piece's last row; the arg-max pairs take a segmented maximum by
-    //    shuffles (the piece's last lane ends with the piece's pair)
-    __syncwarp();  // every lane's row is staged
     const u32 pm = __ballot_sync(0xffffffffu, on && (ed || lane == 31 || tl));  // last lanes of pieces
-    {
-      const bool keep = lane < G && !((am_any >> lane) & 1u);
-      float* col = s.stage + warp * 32 * kQS + lane;
-      const int nv = min(32, np - warp * 32);  // points of this warp (warp-uniform)
-      float a = 0.f;
-      for (int i0 = 0; i0 < nv; i0 += 8) {
-        float x[8];
+    const u32 eb = __ballot_sync(0xffffffffu, ed);
+    int ht = -1;       // tile index of the run's first point (-1: the run began in an earlier tile)
+    int w1 = warp;     // the warp with the run's first piece in the tile
+    int nrun = 0;      // runs that this warp fuses
+    u32 fused = 0;     // the lanes where they end
+    float pb = -INFINITY;  // running arg-max of a class-max source over its segments
+    int pi = 0x7fffffff;
+    const int rounds = MULTI ? s.plan.n_rounds : 1;
+    for (int rd = 0; rd < rounds; ++rd) {
+      const int G = s.plan.ncol[rd];
+      const u32 am_val = s.plan.am[rd], am_any = am_val | (am_val << 1);
+      // B. the point's channels into its row
+      if (on)
+        for (int g = s.plan.seg0[rd]; g < s.plan.seg0[rd + 1]; ++g) {
+          const PlanSeg& sg = s.plan.seg[g];
+          if (TOPK && sg.topk) stage_seg_topk(sg, srow, id, pb, pi);
+          else stage_seg(sg, srow, id, pb, pi);
+          if (sg.cm == 2) {
+            srow[sg.col + sg.n] = pb;
+            srow[sg.col + sg.n + 1] = __int_as_float(pi);
+            pb = -INFINITY;
+            pi = 0x7fffffff;
+          }
+        }
+      u64 zk = 0;  // ray-cast clean-up: (call id, lowest z) key of an accepted point
+      if ((!MULTI || rd == 0) && on) {
+        // C. outlier gate against the pre-call state: the point's height sums
+        const MapCall* mc = md.n_maps > 1 ? job->maps + key / md.W2 : &s.mc0;
+        float z, vm;
+        eval_zvm(md, *mc, xs, ys, zs, z, vm);
+        const bool rej = (fl & kFlagValid) && gate_reject(z, h0, v0, vm, md.lam2);
+        const float w = __frcp_rn(vm);
+        srow[0] = rej ? 0.f : w;
+        srow[1] = rej ? 0.f : z * w;
+        srow[2] = rej ? 0.f : 1.f;
+        srow[3] = rej ? 1.f : 0.f;
+        if (RAY && !rej) zk = call_hi | (u64)(~ordered_bits(__float_as_uint(z)));
+      }
+      // D. sums over the pieces of runs in the warp: lane c walks column c down
+      //    the warp's rows in point order and leaves each piece's sum in the
+      //    piece's last row; the arg-max pairs take a segmented maximum by
+      //    shuffles (the piece's last lane ends with the piece's pair)
+      __syncwarp();  // every lane's row is staged
+      {
+        const bool keep = lane < G && !((am_any >> lane) & 1u);
+        float* col = s.stage + warp * 32 * kQS + lane;
+        const int nv = min(32, np - warp * 32);  // points of this warp (warp-uniform)
+        float a = 0.f;
+        for (int i0 = 0; i0 < nv; i0 += 8) {
+          float x[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) x[u] = col[(i0 + u) * kQS];
+          for (int u = 0; u < 8; ++u) x[u] = col[(i0 + u) * kQS];
+          const u32 ends = (pm >> i0) & 0xffu;
+          if (ends == 0u && i0 + 8 <= nv) {  // no piece ends among these rows
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          if (i0 + u < nv) {
-            a += x[u];
-            if ((pm >> (i0 + u)) & 1u) {
-              if (keep) col[(i0 + u) * kQS] = a;
-              a = 0.f;
+            for (int u = 0; u < 8; ++u) a += x[u];
+          } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              if (i0 + u < nv) {
+                a += x[u];
+                if ((ends >> u) & 1u) {
+                  if (keep) col[(i0 + u) * kQS] = a;
+                  a = 0.f;
+                }
+              }
             }
           }
         }
       }
-    }
-    if (s.n_pair) {
-      bool take[5];
-#pragma unroll
-      for (int k = 0; k < 5; ++k) take[k] = lane - (1 << k) >= hl;
-      for (int k = 0; k < s.n_pair; ++k) {
-        const int c = s.pair_col[k];
+      for (u32 m0 = am_val; m0; m0 &= m0 - 1) {
+        const int c = __ffs(m0) - 1;
         float2 m = make_float2(srow[c], srow[c + 1]);
 #pragma unroll
         for (int b = 0; b < 5; ++b) {
           const float ov = __shfl_up_sync(0xffffffffu, m.x, 1 << b);
           const float oi = __shfl_up_sync(0xffffffffu, m.y, 1 << b);
-          if (take[b]) m = cm_comb(make_float2(ov, oi), m);
+          if (lane - (1 << b) >= hl) m = cm_comb(make_float2(ov, oi), m);
         }
         srow[c] = m.x;
         srow[c + 1] = m.y;
       }
-    }
-    if (RAY) {  // the lowest accepted z of every cell: segmented maximum of the keys, one atomic per piece
+      if (RAY && (!MULTI || rd == 0)) {  // the lowest accepted z of every cell, one atomic per piece
 #pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        const u64 o = __shfl_up_sync(0xffffffffu, zk, 1 << k);
-        if (lane - (1 << k) >= hl && o > zk) zk = o;
-      }
-      if (on && zk != 0 && ((pm >> lane) & 1u)) atomicMax((unsigned long long*)(md.zacc + key), (unsigned long long)zk);
-    }
-    if (t == 0) {  // both slots unused unless a piece below writes one
-      fz_slot(md, acc, tile, 0)[kSlotBits] = 0.f;
-      fz_slot(md, acc, tile, 1)[kSlotBits] = 0.f;
-    }
-    __syncthreads();  // every warp's last row (the piece continuing into the next warp) is complete
-    // E. the lane where a run ends, or where the tile ends inside a run: the
-    //    run's sums over the tile, then the run is fused here or its piece
-    //    goes to a slot
-    if (on && (ed || tl)) {
-      int ht = -1;  // tile index of the run's first point (-1: the run began in an earlier tile)
-      int w1 = warp;
-      if ((hb >> hl) & 1u) {
-        ht = warp * 32 + hl;
-      } else {
-        w1 = 0;
-        for (int w = warp - 1; w >= 0; --w) {
-          const u32 b = s.whd[w];
-          if (b) {
-            ht = w * 32 + 31 - __clz(b);
-            w1 = w;
-            break;
-          }
+        for (int k = 0; k < 5; ++k) {
+          const u64 o = __shfl_up_sync(0xffffffffu, zk, 1 << k);
+          if (lane - (1 << k) >= hl && o > zk) zk = o;
         }
+        if (on && zk != 0 && ((pm >> lane) & 1u)) atomicMax((unsigned long long*)(md.zacc + key), (unsigned long long)zk);
       }
-      if (w1 < warp) {  // the pieces of earlier warps, in warp order, then this lane's piece
-        for (int c = 0; c < G; ++c) {
-          if ((am_val >> c) & 1u) {
-            float2 m = make_float2(s.stage[(w1 * 32 + 31) * kQS + c], s.stage[(w1 * 32 + 31) * kQS + c + 1]);
-            for (int w = w1 + 1; w < warp; ++w)
-              m = cm_comb(m, make_float2(s.stage[(w * 32 + 31) * kQS + c], s.stage[(w * 32 + 31) * kQS + c + 1]));
-            m = cm_comb(m, make_float2(srow[c], srow[c + 1]));
-            srow[c] = m.x;
-            srow[c + 1] = m.y;
-            ++c;
+      if ((!MULTI || rd == 0) && t == 0) {  // both slots unused unless a piece below writes one
+        fz_slot(md, acc, tile, 0)[kSlotBits] = 0.f;
+        fz_slot(md, acc, tile, 1)[kSlotBits] = 0.f;
+      }
+      __syncthreads();  // every warp's last row (the piece continuing into the next warp) is complete
+      if (!MULTI || rd == 0) {
+        // E. where each ended run began in the tile, and the list of the runs fused here
+        if (on && (ed || tl)) {
+          if ((hb >> hl) & 1u) {
+            ht = warp * 32 + hl;
           } else {
-            float a = s.stage[(w1 * 32 + 31) * kQS + c];
-            for (int w = w1 + 1; w < warp; ++w) a += s.stage[(w * 32 + 31) * kQS + c];
-            srow[c] = a + srow[c];
+            w1 = 0;
+            for (int w = warp - 1; w >= 0; --w) {
+              const u32 b = s.whd[w];
+              if (b) {
+                ht = w * 32 + 31 - __clz(b);
+                w1 = w;
+                break;
+              }
+            }
+          }
+        }
+        fused = __ballot_sync(0xffffffffu, ed && ht >= 0);
+        nrun = __popc(fused);
+        if (ed && ht >= 0) {
+          FwRun r;
+          r.g = key;
+          r.fl = fl;
+          r.n = (float)(t - ht + 1);
+          r.row = t;
+          *reinterpret_cast<uint4*>(&s.run[warp][__popc(fused & (le >> 1))]) = *reinterpret_cast<uint4*>(&r);
+        }
+      }
+      // F. a run begun in an earlier warp that ends here (or at the tile's end): it is the
+      //    warp's first piece; the lanes add the earlier warps' pieces, one column each
+      {
+        const int fe = __ffs(pm) - 1;  // last lane of the first piece
+        const bool ends = ((eb >> (fe & 31)) & 1u) || warp * 32 + fe == np - 1;
+        const int wf = __shfl_sync(0xffffffffu, w1, fe & 31);
+        if (fe >= 0 && !(hb & 1u) && ends && wf < warp && lane < G) {
+          float* own = s.stage + (warp * 32 + fe) * kQS + lane;
+          const float* last = s.stage + 31 * kQS + lane;  // last rows of the warps
+          if ((am_val >> lane) & 1u) {
+            float2 m = make_float2(last[wf * 32 * kQS], last[wf * 32 * kQS + 1]);
+            for (int w = wf + 1; w < warp; ++w) m = cm_comb(m, make_float2(last[w * 32 * kQS], last[w * 32 * kQS + 1]));
+            m = cm_comb(m, make_float2(own[0], own[1]));
+            own[0] = m.x;
+            own[1] = m.y;
+          } else if (!((am_any >> lane) & 1u)) {
+            float a = last[wf * 32 * kQS];
+            for (int w = wf + 1; w < warp; ++w) a += last[w * 32 * kQS];
+            own[0] = a + own[0];
           }
         }
       }
-      const u32 nt = (u32)(t - max(ht, 0) + 1);  // points of the run in the tile
-      const u32 g = key;
-      if (ht >= 0 && ed) {
-        // the whole run lies in the tile: every layer's rule, class max, height, flags
-        const float N = (float)nt, rN = __frcp_rn(N);
-        for (int q = 0; q < n_src; ++q)
-          if (s.qn[q] > 0)
-            for (int j = 0; j < s.nrlay[q]; ++j) {
-              const int l = s.rlay[q][j];
-              lane_rule(s.L[l], l, srow + s.qc0[q], s.qch0[q], s.qn[q], g, fl, N, rN);
-            }
-        for (int q = 0; q < n_src; ++q)
-          if (s.src[q].has_classmax) {
-            const int av = s.qc0[q] + s.src[q].C;  // arg-max value column
-            const float best = srow[av];
-            write_classmax(s.L, s.src[q], g, best, best == -INFINITY ? -1 : __float_as_int(srow[av + 1]));
+      __syncwarp();
+      // G. pieces that leave the tile: [0] a run begun in an earlier tile that ends here, [1] a
+      //    run that continues past the tile; lanes over the columns, the header by the piece's lane
+      {
+        const bool piece = on && (ed || tl) && !(ed && ht >= 0);
+        for (u32 pb2 = __ballot_sync(0xffffffffu, piece); pb2; pb2 &= pb2 - 1) {
+          const int l = __ffs(pb2) - 1;
+          float* hdr = fz_slot(md, acc, tile, ((eb >> l) & 1u) ? 0 : 1);
+          if (lane < G) hdr[s.plan.slot[rd * kFuseQ + lane]] = s.stage[(warp * 32 + l) * kQS + lane];
+          if ((!MULTI || rd == 0) && lane == l) {
+            hdr[kSlotKey] = __uint_as_float(key);
+            hdr[kSlotN] = __uint_as_float((u32)(t - max(ht, 0) + 1));
+            hdr[kSlotBits] = __uint_as_float(kBitUsed | (ht >= 0 ? kBitHead : 0u) | (ed ? kBitEnd : 0u));
+            hdr[kSlotFl] = __uint_as_float(fl);
+            hdr[kSlotH0] = h0;
+            hdr[kSlotV0] = v0;
+            hdr[kSlotNacc] = __uint_as_float(na0);
+            hdr[kSlotNrej] = __uint_as_float(nr0);
           }
-        u32 f = fl;
-        height_update(md, g, f, h0, v0, srow[0], srow[1], (u32)srow[2], (u32)srow[3], na0, nr0);
-        for (int q = 0; q < n_src; ++q) {
-          if (any_gauss) write_gauss_var(s.L, s.src[q], g, f, N, rN);
-          for (int b = 0; b < s.src[q].n_layers; ++b) f |= 2u << s.src[q].layers[b];
         }
-        md.flags[g] = f;
-      } else {
-        // [0]: a run begun in an earlier tile that ends here; [1]: a run that continues past the tile
-        float* hdr = fz_slot(md, acc, tile, ed ? 0 : 1);
-        const u32 bits = kBitUsed | (ht >= 0 ? kBitHead : 0u) | (ed ? kBitEnd : 0u);
-        hdr[kSlotKey] = __uint_as_float(g);
-        hdr[kSlotN] = __uint_as_float(nt);
-        hdr[kSlotBits] = __uint_as_float(bits);
-        hdr[kSlotFl] = __uint_as_float(fl);
-        hdr[kSlotH0] = h0;
-        hdr[kSlotV0] = v0;
-        hdr[kSlotNacc] = __uint_as_float(na0);
-        hdr[kSlotNrej] = __uint_as_float(nr0);
-        for (int c = 0; c < G; ++c) hdr[slot_off(c)] = srow[c];
+      }
+      // H. the runs fused here: the round's rules, in round 0 the height
+      run_rules(s, s.run[warp], nrun, s.plan.rule0[rd], s.plan.rule0[rd + 1]);
+      if ((!MULTI || rd == 0) && ((fused >> lane) & 1u)) {
+        u32 f = fl;
+        height_update(md, key, f, h0, v0, srow[0], srow[1], (u32)srow[2], (u32)srow[3], na0, nr0);
+        md.flags[key] = f | s.plan.all_bits;
+      }
+      if (MULTI && rd + 1 < rounds) __syncthreads();  // the next round overwrites the stage
+    }
+    // I. Gaussian variances, after every task read them
+    if (s.plan.n_gauss) {
+      __syncwarp();
+      if ((fused >> lane) & 1u) {
+        const float N = (float)(t - ht + 1);
+        for (int k = 0; k < s.plan.n_gauss; ++k) {
+          float* gv = s.plan.gauss[k].gvar + key;
+          const float var = s.plan.gauss[k].var_meas;
+          if (fl & s.plan.gauss[k].bit) {
+            const float s02 = *gv;
+            *gv = var * s02 * __frcp_rn(__fmaf_rn(N, s02, var));
+          } else {
+            *gv = var * __frcp_rn(N);
+          }
+        }
       }
     }
   }
@@ -1937,6 +2059,13 @@ constexpr int kMaxDevices = 128;
 static int g_sums_ctas_per_sm[kMaxDevices] = {};
 static int g_warps_ctas_per_sm[kMaxDevices] = {};
 
+// the warp fuse kernel by variant: bit 0 top-k rows, bit 1 clean-up stamps, bit 2 several rounds
+using WarpFuseFn = void (*)(MapDev, const PointJob*, int);
+static const WarpFuseFn kWarpFuse[8] = {
+    k_fuse_warps<false, false, false>, k_fuse_warps<true, false, false>, k_fuse_warps<false, true, false>,
+    k_fuse_warps<true, true, false>,   k_fuse_warps<false, false, true>, k_fuse_warps<true, false, true>,
+    k_fuse_warps<false, true, true>,   k_fuse_warps<true, true, true>};
+
 static int current_device() {
   int d = 0;
   if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= kMaxDevices) d = 0;
@@ -1997,16 +2126,10 @@ static cudaError_t launch_rb(Map* m, const PointJob* d_job, cudaStream_t st) {
   {
     ProfScope ps(m, kProfFuseTiles, st);
     const bool topk = m->fuse_variant & 1;
-    if ((m->fuse_variant & 2) && m->tune.fuse_kernel == 0) {  // the columns fit one round: warp kernel
+    if ((m->fuse_variant & 2) && m->tune.fuse_kernel == 0) {  // the call has a plan: warp kernel
       const int cps = g_warps_ctas_per_sm[current_device()];
-      const dim3 grid(sms * (cps > 0 ? cps : 1));
-      const size_t sm = sizeof(WarpSmem);
-      if (topk)
-        md.ray_on ? k_fuse_warps<true, true><<<grid, kFT, sm, st>>>(md, d_job, P & 1)
-                  : k_fuse_warps<true, false><<<grid, kFT, sm, st>>>(md, d_job, P & 1);
-      else
-        md.ray_on ? k_fuse_warps<false, true><<<grid, kFT, sm, st>>>(md, d_job, P & 1)
-                  : k_fuse_warps<false, false><<<grid, kFT, sm, st>>>(md, d_job, P & 1);
+      const int v = (topk ? 1 : 0) | (md.ray_on ? 2 : 0) | ((m->fuse_variant & 4) ? 4 : 0);
+      kWarpFuse[v]<<<dim3(sms * (cps > 0 ? cps : 1)), kFT, sizeof(WarpSmem), st>>>(md, d_job, P & 1);
     } else {
       const int cps = g_sums_ctas_per_sm[current_device()];
       const dim3 grid(sms * (cps > 0 ? cps : 1));
@@ -2042,12 +2165,10 @@ cudaError_t prepare_kernels() {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_sums_ctas_per_sm[dev], k_fuse_tiles<false, false>, kFT,
                                                       sizeof(SumSmem));
   if (g_sums_ctas_per_sm[dev] < 1) g_sums_ctas_per_sm[dev] = 1;
-  for (auto f : {k_fuse_warps<false, false>, k_fuse_warps<false, true>, k_fuse_warps<true, false>,
-                 k_fuse_warps<true, true>})
+  for (auto f : kWarpFuse)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WarpSmem));
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_warps_ctas_per_sm[dev], k_fuse_warps<false, false>, kFT,
-                                                      sizeof(WarpSmem));
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_warps_ctas_per_sm[dev], kWarpFuse[0], kFT, sizeof(WarpSmem));
   if (g_warps_ctas_per_sm[dev] < 1) g_warps_ctas_per_sm[dev] = 1;
   if (e == cudaSuccess) e = set_attrs<8>();
   if (e == cudaSuccess) e = set_attrs<9>();

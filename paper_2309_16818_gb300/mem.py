@@ -366,8 +366,8 @@ class Map:
         _ck(lib().mem_inject_fault(self._h, kind))
 
     def set_tuning(self, radix_bits, blocks_per_sm, fuse_kernel=0):
-        """fuse_kernel 0: per-cell sums in registers where the call's columns fit one round;
-        1: the shared-memory tile kernel always."""
+        """fuse_kernel 0: warps sum and fuse their own points where the call's columns fit the plan;
+        1: the block-wide tile kernel always."""
         _ck(lib().mem_set_tuning(self._h, radix_bits, blocks_per_sm, fuse_kernel))
 
     def get_tuning(self):
