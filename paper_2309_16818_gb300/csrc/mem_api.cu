@@ -1159,7 +1159,7 @@ extern "C" mem_status mem_autotune_batch(mem_map* mm, const int64_t* offsets, co
   cudaError_t ce = copy_all(true);
   const int bits_opts[3] = {8, 9, 10}, bps_opts[3] = {2, 4, 8};
   for (int ki = 0; ki < 6 && ce == cudaSuccess && s == MEM_OK; ++ki) {
-    const int bi = ki % 3, fk = ki / 3;  // both fuse kernels (they differ only where the columns fit one round)
+    const int bi = ki % 3, fk = ki / 3;  // both fuse kernels (they differ only where the warp kernel has a plan)
     const int passes = (m->key_bits + bits_opts[bi] - 1) / bits_opts[bi];
     if (passes > 4) continue;
     for (int pi = 0; pi < 3 && ce == cudaSuccess && s == MEM_OK; ++pi) {

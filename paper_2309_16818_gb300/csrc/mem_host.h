@@ -13,7 +13,7 @@ constexpr int kJobSlots = 8;
 struct Tuning {
   int radix_bits = 9;   // digit width of the radix sort (8..10)
   int blocks_per_sm = 4;
-  int fuse_kernel = 0;   // 0: the warp fuse kernel where a call's columns fit one round; 1: the tile kernel
+  int fuse_kernel = 0;   // 0: the warp fuse kernel where the call has a plan; 1: the tile kernel
 };
 
 struct Map {
