@@ -216,13 +216,17 @@ static cudaError_t dalloc(Map* m, void** p, size_t bytes, bool scratch) {
   return e;
 }
 
+void drop_graphs(Map* m) {
+  for (auto& g : m->graph) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  }
+}
+
 void free_scratch(Map* m) {
   for (void* p : m->scratch_allocs) cudaFree(p);
   m->scratch_allocs.clear();
-  if (m->graph) {
-    cudaGraphExecDestroy(m->graph);
-    m->graph = nullptr;
-  }
+  drop_graphs(m);
 }
 
 cudaError_t alloc_scratch(Map* m, int64_t cap) {
@@ -273,10 +277,7 @@ static cudaError_t ensure_partial(Map* m, int acc) {
   if (e != cudaSuccess) return e;
   md.partial = (float*)p;
   md.partial_cap = need;
-  if (m->graph) {  // the graph captured the old buffer
-    cudaGraphExecDestroy(m->graph);
-    m->graph = nullptr;
-  }
+  drop_graphs(m);
   return cudaSuccess;
 }
 
@@ -388,13 +389,13 @@ static void camera_rel(const double T[16], const double o[2], MapCall& mc) {
 }
 
 // Stage a job block in a pinned slot and queue its copy to the device.
-static mem_status stage_job(Map* m, const void* host, size_t bytes, cudaStream_t st) {
+static mem_status stage_job(Map* m, int jb, const void* host, size_t bytes, cudaStream_t st) {
   if (bytes > m->job_bytes) return fail(MEM_ERR_STATE, "job block too large (%zu bytes)", bytes);
   const int s = m->job_slot;
   m->job_slot = (s + 1) % kJobSlots;
   CK(cudaEventSynchronize(m->job_ev[s]), "cudaEventSynchronize");
   memcpy(m->h_job[s], host, bytes);
-  CK(cudaMemcpyAsync(m->d_job, m->h_job[s], bytes, cudaMemcpyHostToDevice, st), "job upload");
+  CK(cudaMemcpyAsync(m->d_job[jb], m->h_job[s], bytes, cudaMemcpyHostToDevice, st), "job upload");
   CK(cudaEventRecord(m->job_ev[s], st), "cudaEventRecord");
   return MEM_OK;
 }
@@ -537,9 +538,11 @@ extern "C" mem_status mem_create_map(const mem_map_config* cfg, mem_map** out) {
   // job block: header + fuse plan + per-map calls + offsets
   m->job_bytes = sizeof(PointJob) + sizeof(memk::FusePlan) + sizeof(MapCall) * cfg->n_maps +
                  sizeof(int64_t) * (cfg->n_maps + 1) + 64;
-  e = dalloc(m, &p, m->job_bytes, false);
-  if (e != cudaSuccess) return bail(e, "alloc job");
-  m->d_job = (char*)p;
+  for (char*& d : m->d_job) {
+    e = dalloc(m, &p, m->job_bytes, false);
+    if (e != cudaSuccess) return bail(e, "alloc job");
+    d = (char*)p;
+  }
   for (int s2 = 0; s2 < kJobSlots; ++s2) {
     e = cudaMallocHost(&p, m->job_bytes);
     if (e != cudaSuccess) return bail(e, "pinned job slot");
@@ -596,10 +599,7 @@ extern "C" mem_status mem_set_tuning(mem_map* mm, int32_t radix_bits, int32_t bl
   m->tune.fuse_kernel = fuse_kernel;
   m->passes = (m->key_bits + radix_bits - 1) / radix_bits;
   if (m->passes > 4) return fail(MEM_ERR_ARG, "too many radix passes");
-  if (m->graph) {
-    cudaGraphExecDestroy(m->graph);
-    m->graph = nullptr;
-  }
+  drop_graphs(m);
   return MEM_OK;
 }
 
@@ -841,11 +841,12 @@ static mem_status ensure_capacity(Map* m, int64_t n) {
 
 // Builds and uploads the job block, then queues the kernel sequence
 // (replayed from a CUDA graph when `graph` is set and the stream allows it).
-// The job block is uploaded on `job_st` (default: `st`); with `ready` set, the
-// kernels on `st` wait for an event recorded on `job_st` after that upload.
+// The job block goes to device block `jb`, uploaded on `job_st` (default: `st`); with
+// `ready` set, the kernels on `st` wait for an event recorded on `job_st` after that
+// upload (which must itself wait for the last kernels that read block `jb`).
 static mem_status run_points(Map* m, int nm, const int64_t* offsets, int64_t n, const float* xyz,
                              const SrcDev* src, int n_src, const double* T, bool graph, cudaStream_t st,
-                             cudaStream_t job_st = nullptr, cudaEvent_t ready = nullptr) {
+                             cudaStream_t job_st = nullptr, cudaEvent_t ready = nullptr, int jb = kJobDevice) {
   mem_status s = ensure_capacity(m, n);
   if (s != MEM_OK) return s;
   std::string buf(m->job_bytes, '\0');
@@ -871,13 +872,13 @@ static mem_status run_points(Map* m, int nm, const int64_t* offsets, int64_t n, 
   }
   build_fuse_tables(*job, acc, m->cfg);
   build_plan(*plan, *job, m->Lh);
-  job->plan = (const memk::FusePlan*)(m->d_job + plan_at);
+  job->plan = (const memk::FusePlan*)(m->d_job[jb] + plan_at);
   job->plan_vecs = (int)((offsetof(memk::FusePlan, rule) + sizeof(memk::PlanRule) * plan->rule0[plan->n_rounds]) / 16);
   m->fuse_variant = plan->n_rounds == 0 ? 0 : (plan->n_rounds == 1 ? 2 : 6);
   for (int q = 0; q < n_src; ++q) m->fuse_variant |= src[q].topk ? 1 : 0;
-  if (m->graph && m->graph_variant != m->fuse_variant) {  // the graph launches another kernel variant
-    cudaGraphExecDestroy(m->graph);
-    m->graph = nullptr;
+  if (m->graph[jb] && m->graph_variant[jb] != m->fuse_variant) {  // the graph launches another kernel variant
+    cudaGraphExecDestroy(m->graph[jb]);
+    m->graph[jb] = nullptr;
   }
   acc = (acc + 3) / 4 * 4;  // slots start on 16-byte boundaries (vector loads of their headers)
   job->acc = acc;
@@ -886,8 +887,8 @@ static mem_status run_points(Map* m, int nm, const int64_t* offsets, int64_t n, 
     if (e != cudaSuccess) return cuda_fail(e, "partial-record buffer");
   }
   if (((uintptr_t)m->md.partial & 15) != 0) return fail(MEM_ERR_STATE, "fuse scratch not 16-byte aligned");
-  job->maps = (const MapCall*)(m->d_job + maps_at);
-  job->offsets = nm > 1 ? (const int64_t*)(m->d_job + offs_at) : nullptr;
+  job->maps = (const MapCall*)(m->d_job[jb] + maps_at);
+  job->offsets = nm > 1 ? (const int64_t*)(m->d_job[jb] + offs_at) : nullptr;
   for (int b = 0; b < nm; ++b) {
     memset(&mcs[b], 0, sizeof(MapCall));
     pose_rel(T + 16 * b, &m->origin[2 * b], mcs[b]);
@@ -899,7 +900,7 @@ static mem_status run_points(Map* m, int nm, const int64_t* offsets, int64_t n, 
     for (int b = 0; b <= nm; ++b) offs[b] = offsets[b];
     bytes = offs_at + sizeof(int64_t) * (nm + 1);
   }
-  s = stage_job(m, h, bytes, ready ? job_st : st);
+  s = stage_job(m, jb, h, bytes, ready ? job_st : st);
   if (s != MEM_OK) return s;
   if (ready) {
     CK(cudaEventRecord(ready, job_st), "job upload record");
@@ -915,22 +916,22 @@ static mem_status run_points(Map* m, int nm, const int64_t* offsets, int64_t n, 
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (graph && st) cudaStreamIsCapturing(st, &cap);
   if (graph && st && cap == cudaStreamCaptureStatusNone && m->use_graph && !m->prof_on) {
-    if (!m->graph) {
+    if (!m->graph[jb]) {
       cudaGraph_t gph;
       CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "begin capture");
-      cudaError_t e = launch_point_fuse(m, (const PointJob*)m->d_job, st);
+      cudaError_t e = launch_point_fuse(m, (const PointJob*)m->d_job[jb], st);
       cudaError_t e2 = cudaStreamEndCapture(st, &gph);
       if (e != cudaSuccess) return cuda_fail(e, "capture launch");
       if (e2 != cudaSuccess) return cuda_fail(e2, "end capture");
-      e = cudaGraphInstantiate(&m->graph, gph, 0);
+      e = cudaGraphInstantiate(&m->graph[jb], gph, 0);
       cudaGraphDestroy(gph);
       if (e != cudaSuccess) return cuda_fail(e, "graph instantiate");
-      m->graph_variant = m->fuse_variant;
+      m->graph_variant[jb] = m->fuse_variant;
     }
-    CK(cudaGraphLaunch(m->graph, st), "graph launch");
+    CK(cudaGraphLaunch(m->graph[jb], st), "graph launch");
     return MEM_OK;
   }
-  CK(launch_point_fuse(m, (const PointJob*)m->d_job, st), "point fuse launch");
+  CK(launch_point_fuse(m, (const PointJob*)m->d_job[jb], st), "point fuse launch");
   return MEM_OK;
 }
 
@@ -1015,9 +1016,10 @@ extern "C" mem_status mem_fuse_pointcloud_host(mem_map* mm, int64_t n, const flo
       src[q].vec_ok = !src[q].topk;  // 256-byte aligned
     }
   }
-  // the job block follows the inputs on the copy stream; the kernels wait for both
+  // the job block (this buffer's: the previous call's kernels may still read theirs) follows the
+  // inputs on the copy stream; the kernels wait for both
   s = run_points(m, 1, nullptr, n, (const float*)(d + off[0]), src, n_sources, T_map_sensor, true, st,
-                 m->copy_stream, m->stage_copied[k]);
+                 m->copy_stream, m->stage_copied[k], k);
   if (s != MEM_OK) return s;
   CK(cudaEventRecord(m->stage_done[k], st), "staging record");
   return MEM_OK;
@@ -1168,10 +1170,7 @@ extern "C" mem_status mem_autotune_batch(mem_map* mm, const int64_t* offsets, co
       m->tune.blocks_per_sm = bps_opts[pi];
       m->tune.fuse_kernel = fk;
       m->passes = passes;
-      if (m->graph) {
-        cudaGraphExecDestroy(m->graph);
-        m->graph = nullptr;
-      }
+      drop_graphs(m);
       float acc_ms = 0.f;
       for (int r = 0; r <= reps && s == MEM_OK; ++r) {  // r = 0 warms up (and captures the graph)
         if ((ce = copy_all(false)) != cudaSuccess) break;
@@ -1197,10 +1196,7 @@ extern "C" mem_status mem_autotune_batch(mem_map* mm, const int64_t* offsets, co
   m->tune = (s == MEM_OK && ce == cudaSuccess) ? best_t : saved;
   m->passes = (s == MEM_OK && ce == cudaSuccess) ? (m->key_bits + m->tune.radix_bits - 1) / m->tune.radix_bits
                                                  : saved_passes;
-  if (m->graph) {
-    cudaGraphExecDestroy(m->graph);
-    m->graph = nullptr;
-  }
+  drop_graphs(m);
   cudaError_t ce2 = copy_all(false);
   cudaStreamSynchronize(st);
   cudaFree(backup);

@@ -9,6 +9,7 @@
 namespace memh {
 
 constexpr int kJobSlots = 8;
+constexpr int kJobBlocks = 3, kJobDevice = 2;  // device job blocks; the one of calls on device buffers
 
 struct Tuning {
   int radix_bits = 9;   // digit width of the radix sort (8..10)
@@ -27,20 +28,21 @@ struct Map {
   // fuse kernel variant of the current point-path call: bit 0 a source has top-k rows,
   // bit 1 it fits the warp kernel's plan (else the tile kernel runs), bit 2 in several rounds
   int fuse_variant = 0;
-  int graph_variant = -1;  // the variant the captured graph launches
   int n_sm = 148;
   int device = 0;
   std::vector<double> origin;  // [n_maps][2] world xy of each map centre
   std::vector<int> ring;       // [n_maps][2] ring-buffer offsets (physical = logical + ring mod W)
   // device job block and pinned staging slots
-  char* d_job = nullptr;
+  // (one per staging buffer of the host path, whose job follows its inputs on the copy stream while
+  // the previous call's kernels still read theirs, and one for calls on device buffers)
+  char* d_job[kJobBlocks] = {};
   size_t job_bytes = 0;
   char* h_job[kJobSlots] = {};
   cudaEvent_t job_ev[kJobSlots] = {};
   int job_slot = 0;
-  // CUDA graph of the batched point path
-  cudaGraphExec_t graph = nullptr;
-  cudaStream_t graph_stream = nullptr;
+  // CUDA graphs of the point path, one per job block, and the fuse kernel variant each launches
+  cudaGraphExec_t graph[kJobBlocks] = {};
+  int graph_variant[kJobBlocks] = {-1, -1, -1};
   bool use_graph = true;
   // optional per-kernel timing (CUDA events around each launch group)
   bool prof_on = false;
@@ -104,6 +106,8 @@ struct ProfScope {
   }
 };
 
+// the graphs hold the map's buffers and schedule: dropped whenever one of these changes
+void drop_graphs(Map* m);
 cudaError_t alloc_scratch(Map* m, int64_t cap);
 void free_scratch(Map* m);
 int key_bits_for(const Map* m);
