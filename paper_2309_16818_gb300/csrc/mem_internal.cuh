@@ -456,6 +456,15 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
+// Programmatic dependent launch of the point path's kernel sequence: a kernel may become
+// resident while the last blocks of the previous one end, and waits for that kernel to
+// have finished, with its writes visible, before it reads anything but the call's job
+// (uploaded before the sequence's first kernel, which is launched the ordinary way). What
+// an earlier kernel of the sequence wrote is never read through the read-only path
+// (__ldg), which assumes data that do not change while the kernel is resident. A no-op
+// for ordinary launches.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // relaxed device-scope loads/stores for the radix-sort look-back
 __device__ __forceinline__ u32 ld_relaxed(const u32* p) {
   u32 v;

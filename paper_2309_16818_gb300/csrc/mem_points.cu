@@ -144,6 +144,7 @@ __global__ void __launch_bounds__(256) k_points_key(MapDev md, const PointJob* _
 //    float32(alpha * mean) when enough points entered it
 
 __global__ void __launch_bounds__(256) k_drift_reduce(MapDev md, const PointJob* __restrict__ job) {
+  pdl_wait();
   if (*(volatile int*)md.err) return;  // a device error is pending: the point path does nothing
   const int b = blockIdx.y, r = blockIdx.x;
   int64_t o0 = 0, o1 = job->n;
@@ -186,6 +187,7 @@ __global__ void __launch_bounds__(256) k_drift_reduce(MapDev md, const PointJob*
 }
 
 __global__ void __launch_bounds__(256) k_drift_apply(MapDev md) {
+  pdl_wait();
   if (*(volatile int*)md.err) return;  // a device error is pending: the point path does nothing
   const int b = blockIdx.y;
   __shared__ float s_shift;
@@ -239,6 +241,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(MapDev md, const P
   __shared__ u32 s_wsum[WARPS];
   __shared__ volatile int s_fail;  // a look-back wait of this tile ran out: no scatter
 
+  pdl_wait();
   // a device error is pending (the word can be set by other blocks of this pass meanwhile, so the
   // block decides once, through shared memory): the point path does nothing
   if (threadIdx.x == 0) s_fail = *(volatile int*)md.err;
@@ -248,9 +251,9 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(MapDev md, const P
   const int64_t n = job->n;
   const int n_tiles = (int)((n + kTile - 1) / kTile);
   const int shift = pass * RB;
-  const u32* __restrict__ kin = (pass & 1) ? md.keys1 : md.keys0;
+  const u32* kin = (pass & 1) ? md.keys1 : md.keys0;
   u32* __restrict__ kout = (pass & 1) ? md.keys0 : md.keys1;
-  const u32* __restrict__ vin = (pass & 1) ? md.vals1 : md.vals0;
+  const u32* vin = (pass & 1) ? md.vals1 : md.vals0;
   u32* __restrict__ vout = (pass & 1) ? md.vals0 : md.vals1;
   u32* lb = md.lookback + (size_t)pass * md.cap_tiles * RADIX;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -294,8 +297,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(MapDev md, const P
     for (int j = 0; j < kSortItems; ++j) {
       const int64_t idx = wbase + j * 32 + lane;
       const bool ok = idx < n;
-      key[j] = ok ? kin[idx] : 0xffffffffu;
-      val[j] = ok ? (pass == 0 ? (u32)idx : vin[idx]) : 0u;
+      key[j] = ok ? __ldcg(kin + idx) : 0xffffffffu;
+      val[j] = ok ? (pass == 0 ? (u32)idx : __ldcg(vin + idx)) : 0u;
     }
     // ranks within the warp, in (item, lane) order = input order
 #pragma unroll
@@ -860,9 +863,10 @@ __global__ void __launch_bounds__(kFT, 7) k_fuse_tiles(MapDev md, const PointJob
                                                        int sorted1) {
   extern __shared__ __align__(16) unsigned char fz_raw[];
   SumSmem& s = *reinterpret_cast<SumSmem*>(fz_raw);
+  pdl_wait();
   if (*(volatile int*)md.err) return;  // a device error is pending: the point path does nothing
-  const u32* __restrict__ sk = sorted1 ? md.keys1 : md.keys0;
-  const u32* __restrict__ sv = sorted1 ? md.vals1 : md.vals0;
+  const u32* sk = sorted1 ? md.keys1 : md.keys0;
+  const u32* sv = sorted1 ? md.vals1 : md.vals0;
   const int64_t n_kept = *(volatile u32*)&md.counters[6];
   const int n_tiles = (int)((n_kept + kFT - 1) / kFT);
   const int n_src = job->n_src;
@@ -904,11 +908,11 @@ __global__ void __launch_bounds__(kFT, 7) k_fuse_tiles(MapDev md, const PointJob
     const int np = (int)min((int64_t)kFT, n_kept - p0);
     // A. keys, point indices, runs
     if (t < np) {
-      s.key[t + 1] = sk[p0 + t];
-      s.idx[t] = sv[p0 + t];
+      s.key[t + 1] = __ldcg(sk + p0 + t);
+      s.idx[t] = __ldcg(sv + p0 + t);
     }
-    if (t == 0) s.key[0] = p0 > 0 ? sk[p0 - 1] : 0xfffffffeu;
-    if (t == 32) s.key[np + 1] = (p0 + np < n_kept) ? sk[p0 + np] : 0xfffffffeu;
+    if (t == 0) s.key[0] = p0 > 0 ? __ldcg(sk + p0 - 1) : 0xfffffffeu;
+    if (t == 32) s.key[np + 1] = (p0 + np < n_kept) ? __ldcg(sk + p0 + np) : 0xfffffffeu;
     __syncthreads();
     const bool hd = t < np && (t == 0 || s.key[t] != s.key[t + 1]);
     const bool ed = t < np && (t == np - 1 || s.key[t + 1] != s.key[t + 2]);
@@ -1606,16 +1610,12 @@ __global__ void __launch_bounds__(kFT, kWarpBlocks) k_fuse_warps(MapDev md, cons
                                                                  int sorted1) {
   extern __shared__ __align__(16) unsigned char fw_raw[];
   WarpSmem& s = *reinterpret_cast<WarpSmem*>(fw_raw);
-  if (*(volatile int*)md.err) return;  // a device error is pending: the point path does nothing
-  const u32* __restrict__ sk = sorted1 ? md.keys1 : md.keys0;
-  const u32* __restrict__ sv = sorted1 ? md.vals1 : md.vals0;
-  const int64_t n_kept = *(volatile u32*)&md.counters[6];
-  const int n_tiles = (int)((n_kept + kFT - 1) / kFT);
+  const u32* sk = sorted1 ? md.keys1 : md.keys0;
+  const u32* sv = sorted1 ? md.vals1 : md.vals0;
   const int acc = job->acc;
   const float* __restrict__ xyz = job->xyz;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const u64 call_hi = RAY ? (u64)job->call_id << 32 : 0ull;
-  if (blockIdx.x >= n_tiles) return;
   // the call's plan (built on the host) into shared memory
   if (job->plan) {
     const uint4* ps = reinterpret_cast<const uint4*>(job->plan);
@@ -1634,6 +1634,11 @@ __global__ void __launch_bounds__(kFT, kWarpBlocks) k_fuse_warps(MapDev md, cons
     }
   }
   if (t == 0) s.mc0 = job->maps[0];
+  pdl_wait();
+  if (*(volatile int*)md.err) return;  // a device error is pending: the point path does nothing
+  const int64_t n_kept = *(volatile u32*)&md.counters[6];
+  const int n_tiles = (int)((n_kept + kFT - 1) / kFT);
+  if (blockIdx.x >= n_tiles) return;
   const u32 le = 0xffffffffu >> (31 - lane);  // lanes up to this one
   u32 heads = 0;  // runs that begin at this thread's points
   float* srow = s.stage + t * kQS;
@@ -1645,10 +1650,10 @@ __global__ void __launch_bounds__(kFT, kWarpBlocks) k_fuse_warps(MapDev md, cons
     // A. key, neighbours' keys, runs and pieces
     u32 key = 0xfffffffeu, kprev = 0xfffffffeu, knext = 0xfffffffeu, id = 0;
     if (on) {
-      key = sk[p];
-      id = sv[p];
-      if (p > 0) kprev = sk[p - 1];
-      if (p + 1 < n_kept) knext = sk[p + 1];
+      key = __ldcg(sk + p);
+      id = __ldcg(sv + p);
+      if (p > 0) kprev = __ldcg(sk + p - 1);
+      if (p + 1 < n_kept) knext = __ldcg(sk + p + 1);
     }
     __syncthreads();  // plan in place; the previous tile is done with the shared arrays
     const bool hd = on && key != kprev;  // a run begins here
@@ -1890,12 +1895,9 @@ __global__ void __launch_bounds__(kFT, kWarpBlocks) k_fuse_warps(MapDev md, cons
 // column over the pieces in tile order and loads the old values of the
 // column's layers together, then stores the new values.
 __global__ void __launch_bounds__(128) k_fuse_cross(MapDev md, const PointJob* __restrict__ job) {
-  if (*(volatile int*)md.err) return;  // a device error is pending: the point path does nothing
   __shared__ LayerDev sL[kMaxLayers];
   __shared__ SrcDev ssrc[kMaxSources];
   __shared__ int srlay[kMaxSources][kMaxSrcLayers], snrlay[kMaxSources];
-  const int64_t n_kept = *(volatile u32*)&md.counters[6];
-  const int n_tiles = (int)((n_kept + kFT - 1) / kFT);
   const int n_src = job->n_src;
   const int acc = job->acc;
   const int G = job->ft.ncol;
@@ -1906,6 +1908,10 @@ __global__ void __launch_bounds__(128) k_fuse_cross(MapDev md, const PointJob* _
     snrlay[t] = job->ft.nrlay[t];
     for (int b = 0; b < kMaxSrcLayers; ++b) srlay[t][b] = job->ft.rlay[t][b];
   }
+  pdl_wait();
+  if (*(volatile int*)md.err) return;  // a device error is pending: the point path does nothing
+  const int64_t n_kept = *(volatile u32*)&md.counters[6];
+  const int n_tiles = (int)((n_kept + kFT - 1) / kFT);
   __syncthreads();
   const int lane = t & 31;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -1959,6 +1965,7 @@ __global__ void __launch_bounds__(128) k_fuse_cross(MapDev md, const PointJob* _
 constexpr int kRayThreads = 128;
 
 __global__ void __launch_bounds__(kRayThreads) k_raycast(MapDev md, const PointJob* __restrict__ job) {
+  pdl_wait();
   if (*(volatile int*)md.err) return;  // a device error is pending: the point path does nothing
   const int W = md.W;
   const int b = blockIdx.y;
@@ -1973,10 +1980,10 @@ __global__ void __launch_bounds__(kRayThreads) k_raycast(MapDev md, const PointJ
   __syncthreads();
   const u32 call = job->call_id;
   const u32 base = (u32)b * md.W2;
-  const u32* __restrict__ stamp = reinterpret_cast<const u32*>(md.zacc);  // [2g + 1]: call id of cell g
+  const u32* stamp = reinterpret_cast<const u32*>(md.zacc);  // [2g + 1]: call id of cell g
   const u32 pair = threadIdx.x * gridDim.x + blockIdx.x;
   if (pair < md.W2 / 2) {  // W is even: a pair lies in one row
-    const ulonglong2 v2 = __ldg(reinterpret_cast<const ulonglong2*>(md.zacc + base + 2 * pair));
+    const ulonglong2 v2 = *reinterpret_cast<const ulonglong2*>(md.zacc + base + 2 * pair);
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const u64 v = u ? v2.y : v2.x;
@@ -2015,8 +2022,8 @@ __global__ void __launch_bounds__(kRayThreads) k_raycast(MapDev md, const PointJ
         const bool act = lw.next(qx[u], qy[u]);
         q[u] = base + phys_cell(md, smc, act ? qx[u] : sx, act ? qy[u] : sy);
         fl[u] = act ? md.flags[q[u]] : 0u;
-        st[u] = act ? __ldg(stamp + 2 * (size_t)q[u] + 1) : call;
-        hq[u] = act ? __ldg(md.h + q[u]) : 0.f;
+        st[u] = act ? stamp[2 * (size_t)q[u] + 1] : call;
+        hq[u] = act ? md.h[q[u]] : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < kRayU; ++u) {
@@ -2038,6 +2045,7 @@ __global__ void __launch_bounds__(kRayThreads) k_raycast(MapDev md, const PointJ
 
 // time-dependent variance growth of every valid cell
 __global__ void k_time_update(MapDev md, int64_t cells) {
+  pdl_wait();
   if (*(volatile int*)md.err) return;  // a device error is pending: the point path does nothing
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < cells;
        g += (int64_t)gridDim.x * blockDim.x)
@@ -2089,14 +2097,41 @@ static cudaError_t set_attrs() {
   return e;
 }
 
-cudaError_t launch_time_update(Map* m, cudaStream_t st) {
+// A launch of the point path's sequence behind its predecessor: outside a capture as a
+// programmatic dependent launch (see pdl_wait), so that the launch, the start of the
+// blocks and their reads of the job overlap the previous kernel's end. Four calls of
+// 131k points on caller-owned layers (seven launches each): 239 -> 186 us. Inside a
+// graph, whose kernels follow one another closely anyway, it gains nothing (three poses 376
+// us either way, with clean-up 390 -> 400 us), nor does letting the next kernel start
+// before the blocks end (its blocks take shared memory from the running kernel's:
+// 199, 378, 424 us).
+template <typename... P, typename... A>
+static cudaError_t launch_next(void (*k)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, bool pdl,
+                               A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
+// time-dependent variance growth; `pdl`: it follows a kernel of the point path
+static cudaError_t time_update(Map* m, cudaStream_t st, bool pdl) {
   const MapDev& md = m->md;
   if (md.time_var == 0.f) return cudaSuccess;
   ProfScope ps(m, kProfTime, st);
   const int64_t cells = (int64_t)md.n_maps * md.W2;
-  k_time_update<<<m->n_sm * m->tune.blocks_per_sm, 256, 0, st>>>(md, cells);
-  return cudaGetLastError();
+  const unsigned grid = (unsigned)(m->n_sm * m->tune.blocks_per_sm);
+  return launch_next(k_time_update, dim3(grid), 256, 0, st, pdl, md, cells);
 }
+
+cudaError_t launch_time_update(Map* m, cudaStream_t st) { return time_update(m, st, false); }
 
 template <int RB>
 static cudaError_t launch_rb(Map* m, const PointJob* d_job, cudaStream_t st) {
@@ -2113,15 +2148,22 @@ static cudaError_t launch_rb(Map* m, const PointJob* d_job, cudaStream_t st) {
     ProfScope ps(m, kProfKey, st);
     k_points_key<RB><<<sms * bps, 256, sizeof(u32) * (P * (1 << RB) + 1), st>>>(md, d_job, P);
   }
+  e = cudaGetLastError();
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (e == cudaSuccess && st) e = cudaStreamIsCapturing(st, &cap);  // (the default stream cannot be captured)
+  const bool pdl = cap == cudaStreamCaptureStatusNone;
+  auto next = [&](auto k, dim3 grid, unsigned block, size_t smem, auto... args) {
+    if (e == cudaSuccess) e = launch_next(k, grid, block, smem, st, pdl, args...);
+  };
   if (md.drift_alpha != 0.0) {
     ProfScope ps(m, kProfDrift, st);
-    k_drift_reduce<<<dim3(md.drift_R, md.n_maps), 256, 0, st>>>(md, d_job);
+    next(k_drift_reduce, dim3(md.drift_R, md.n_maps), 256, 0, md, d_job);
     const u32 per_map = (md.W2 + 256 * 8 - 1) / (256 * 8);
-    k_drift_apply<<<dim3(per_map, md.n_maps), 256, 0, st>>>(md);
+    next(k_drift_apply, dim3(per_map, md.n_maps), 256, 0, md);
   }
   {
     ProfScope ps(m, kProfSort, st);
-    for (int p = 0; p < P; ++p) k_onesweep<RB><<<sms * 2, kSortThreads, sort_smem<RB>(), st>>>(md, d_job, p);
+    for (int p = 0; p < P; ++p) next(k_onesweep<RB>, dim3(sms * 2), kSortThreads, sort_smem<RB>(), md, d_job, p);
   }
   {
     ProfScope ps(m, kProfFuseTiles, st);
@@ -2129,30 +2171,26 @@ static cudaError_t launch_rb(Map* m, const PointJob* d_job, cudaStream_t st) {
     if ((m->fuse_variant & 2) && m->tune.fuse_kernel == 0) {  // the call has a plan: warp kernel
       const int cps = g_warps_ctas_per_sm[current_device()];
       const int v = (topk ? 1 : 0) | (md.ray_on ? 2 : 0) | ((m->fuse_variant & 4) ? 4 : 0);
-      kWarpFuse[v]<<<dim3(sms * (cps > 0 ? cps : 1)), kFT, sizeof(WarpSmem), st>>>(md, d_job, P & 1);
+      next(kWarpFuse[v], dim3(sms * (cps > 0 ? cps : 1)), kFT, sizeof(WarpSmem), md, d_job, P & 1);
     } else {
       const int cps = g_sums_ctas_per_sm[current_device()];
       const dim3 grid(sms * (cps > 0 ? cps : 1));
-      if (topk)
-        md.ray_on ? k_fuse_tiles<true, true><<<grid, kFT, sizeof(SumSmem), st>>>(md, d_job, P & 1)
-                  : k_fuse_tiles<true, false><<<grid, kFT, sizeof(SumSmem), st>>>(md, d_job, P & 1);
-      else
-        md.ray_on ? k_fuse_tiles<false, true><<<grid, kFT, sizeof(SumSmem), st>>>(md, d_job, P & 1)
-                  : k_fuse_tiles<false, false><<<grid, kFT, sizeof(SumSmem), st>>>(md, d_job, P & 1);
+      next(topk ? (md.ray_on ? k_fuse_tiles<true, true> : k_fuse_tiles<true, false>)
+                : (md.ray_on ? k_fuse_tiles<false, true> : k_fuse_tiles<false, false>),
+           grid, kFT, sizeof(SumSmem), md, d_job, P & 1);
     }
   }
   {
     ProfScope ps(m, kProfFuseCross, st);
-    k_fuse_cross<<<sms * 8, 128, 0, st>>>(md, d_job);
+    next(k_fuse_cross, dim3(sms * 8), 128, 0, md, d_job);
   }
   if (md.ray_on) {
     ProfScope ps(m, kProfRay, st);
     const u32 pairs = md.W2 / 2;
-    k_raycast<<<dim3((pairs + kRayThreads - 1) / kRayThreads, md.n_maps), kRayThreads, 0, st>>>(md, d_job);
+    next(k_raycast, dim3((pairs + kRayThreads - 1) / kRayThreads, md.n_maps), kRayThreads, 0, md, d_job);
   }
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_time_update(m, st);
+  return time_update(m, st, pdl);
 }
 
 cudaError_t prepare_kernels() {
