@@ -1,7 +1,11 @@
 // Learned inpainting: a small U-Net trained and run with BF16 tensor-core
 // kernels (float32 accumulation, float32 master weights, Adam).
 //
-// Layout: activations NHWC bf16. A 3x3 convolution is an implicit GEMM
+// Layout: activations are bf16 in planes of 8 channels, [n][c / 8][h][w][8], so that a
+// row of a halo box is one run of 16 bytes per pixel (with [n][h][w][c] every pixel of
+// a box was a separate 16-byte request, and these set the pace of the full-resolution
+// layers), an epilogue's store instruction writes whole 128-byte rows of a tile, and
+// what works on pixels of 8 channels takes a tensor as n c / 8 images. A 3x3 convolution is an implicit GEMM
 // C[pixels, cout] = A[pixels, 9*cin] B[9*cin, cout] on the tcgen05 tensor
 // cores: TMA box loads bring the input halo of a 16 x 16 output tile (16
 // channels per pipeline stage, zero outside the image) and one bulk copy the
@@ -18,6 +22,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "mem_host.h"
@@ -121,17 +126,17 @@ __device__ __forceinline__ void tmem_ld16(u32 taddr, u32 v[16]) {
 // 3x3 convolution (forward, and data gradient with flipped weights)
 
 struct ConvArgs {
-  const bf16* in0;  // [N, H(/2), W(/2), c0]
-  const bf16* in1;  // [N, H, W, c1] or null
+  const bf16* in0;  // N images of c0 channels, at half resolution if up0
+  const bf16* in1;  // N images of c1 channels, or null
   int c0, c1, up0;  // up0: in0 is at half resolution (nearest upsample)
   int cin_pad;      // input channels of the packed weights (multiple of 16, >= c0 + c1)
   const bf16* w;    // packed [cout / BN][cin_pad / 16][9 taps][2][BN][8] (see conv_bn)
   const float* bias;
-  bf16* out;        // [N, H, W, cout]
+  bf16* out;        // N images of cout channels
   int cout, N, H, W, relu;
   int* err;         // set when a bounded wait runs out
   int store;        // write `out` (0: only the fused outputs below are wanted)
-  bf16* pool;       // optional 2x2 max pooling of the output, [N, H/2, W/2, cout]
+  bf16* pool;       // optional 2x2 max pooling of the output, at half resolution
   // optional fused 1x1 head (one column block only): pred = fill + head_b + sum_c head_w[c] out[c]
   const float* head_w;
   const float* head_b;
@@ -147,8 +152,8 @@ __host__ __device__ inline int conv_bn(int cout) { return cout % 128 == 0 ? 128 
 // accumulates in TMEM as two M = 128 halves (16 rows x 8 columns of pixels
 // each), K = 9 taps x the input channels. The input is consumed 16 channels
 // per pipeline stage: the 18 x 18 halo of the tile arrives in shared memory
-// as two planes of 8 channels (16 bytes per pixel) by two TMA box loads,
-// which read zero outside the image, so the 8-pixel rows of a tap's A operand
+// as two planes of 8 channels (16 bytes per pixel) by one TMA box load,
+// which reads zero outside the image, so the 8-pixel rows of a tap's A operand
 // are eight consecutive 16-byte halo pixels: every tap reads the same halo
 // through a descriptor offset by (dy * 18 + dx) pixels, with 288 bytes between
 // pixel rows and one plane between the two 8-channel halves of K. The
@@ -169,11 +174,9 @@ __host__ __device__ inline int conv_bn(int cout) { return cout % 128 == 0 ? 128 
 // (128 epilogue arrivals). Every wait is bounded.
 constexpr int kTY = 16, kTX = 16;              // output tile
 constexpr int kHY = kTY + 2, kHX = kTX + 2;    // input halo
-constexpr int kPlaneBytes = kHY * kHX * 16;    // one 8-channel halo plane as loaded (5184)
-constexpr int kPlane = 5248;                   // its stride in shared memory (128-byte multiple)
+constexpr int kPlane = kHY * kHX * 16;         // bytes of one 8-channel halo plane (5184)
 constexpr int kHalfBox = 10;                   // half-resolution box side for upsampled input
-constexpr int kStgBytes = kHalfBox * kHalfBox * 16;  // one plane of it (1600)
-constexpr int kStg = 1664;                     // its stride in shared memory
+constexpr int kStg = kHalfBox * kHalfBox * 16; // bytes of one plane of it (1600)
 constexpr int kConvProd = 96;                  // gathering threads (warps 1..3)
 constexpr int kConvEpi = 128;                  // epilogue threads (warps 4..7)
 
@@ -181,6 +184,7 @@ template <int BN, int NST>
 struct ConvCfg {
   static constexpr int kWBytes = 9 * 2 * BN * 16;             // weights of one stage
   static constexpr int kSlot = 2 * kPlane + kWBytes + 2 * kStg;  // one pipeline slot
+  static_assert(kSlot % 128 == 0 && (2 * kPlane) % 128 == 0 && kWBytes % 128 == 0, "TMA boxes start on 128 bytes");
   static constexpr int kSmem = NST * kSlot + 256 + 2048 + 1024;  // + barriers, bias and head, slack
   static constexpr int kCols = 4 * BN;                        // TMEM columns: 2 buffers x 2 halves
   static constexpr int kMaxBlocksPerSm = 512 / kCols;         // TMEM holds 512 columns
@@ -297,16 +301,14 @@ __global__ void __launch_bounds__(256, ConvCfg<BN, NST>::kMaxBlocksPerSm)
         const CUtensorMap* map = from0 ? &tm0 : &tm1;
         const int c = from0 ? cb : cb - a.c0;
         if (pt == 0) {
-          const u32 bytes = C::kWBytes + (up ? 0u : 2u * kPlaneBytes);
+          const u32 bytes = C::kWBytes + (up ? 0u : 2u * kPlane);
           mbar_arrive_tx(full0 + 8 * slot, bytes);
           bulk_g2s(wb, a.w + (int64_t)(nb * CS + s) * (9 * 2 * BN * 8), C::kWBytes, full0 + 8 * slot);
           if (up) {
-            mbar_arrive_tx(stg0 + 8 * slot, 2u * kStgBytes);
-            tma_load_4d(sb, map, c, (x0 >> 1) - 1, (y0 >> 1) - 1, n, stg0 + 8 * slot);
-            tma_load_4d(sb + kStg, map, c + 8, (x0 >> 1) - 1, (y0 >> 1) - 1, n, stg0 + 8 * slot);
+            mbar_arrive_tx(stg0 + 8 * slot, 2u * kStg);
+            tma_load_4d(sb, map, ((x0 >> 1) - 1) * 8, (y0 >> 1) - 1, c >> 3, n, stg0 + 8 * slot);
           } else {
-            tma_load_4d(hb, map, c, x0 - 1, y0 - 1, n, full0 + 8 * slot);
-            tma_load_4d(hb + kPlane, map, c + 8, x0 - 1, y0 - 1, n, full0 + 8 * slot);
+            tma_load_4d(hb, map, (x0 - 1) * 8, y0 - 1, c >> 3, n, full0 + 8 * slot);
           }
         }
         if (up) {
@@ -352,13 +354,14 @@ __global__ void __launch_bounds__(256, ConvCfg<BN, NST>::kMaxBlocksPerSm)
       for (int h = 0; h < 2; ++h) {
         const int yy = y0 + (m >> 3), xx = x0 + 8 * h + (m & 7);
         const bool inside = yy < a.H && xx < a.W;
-        const int64_t pix = ((int64_t)n * a.H + (inside ? yy : 0)) * a.W + (inside ? xx : 0);
-        bf16* o = a.out + pix * a.cout + nb * BN;
+        const int64_t hw = (int64_t)a.H * a.W, at = inside ? (int64_t)yy * a.W + xx : 0;
+        const int64_t pix = (int64_t)n * hw + at;
+        bf16* o = a.out + (((int64_t)n * a.cout + nb * BN) * hw + at * 8);  // plane c / 8 at c hw
         // pooling partners: lanes ^1 (x + 1) and ^8 (y + 1); lane bits 0 and 3 clear = top-left
         // pixel, and H, W are even wherever pooling happens, so a window is wholly inside or outside
         const bool pool_writer = inside && (lane & 9) == 0;
-        bf16* po = a.pool ? a.pool + (((int64_t)n * (a.H >> 1) + (yy >> 1)) * (a.W >> 1) + (xx >> 1)) * a.cout +
-                                nb * BN
+        bf16* po = a.pool ? a.pool + (((int64_t)n * a.cout + nb * BN) * (hw >> 2) +
+                                      ((int64_t)(yy >> 1) * (a.W >> 1) + (xx >> 1)) * 8)
                           : nullptr;
         float hr = a.head_w ? a.head_b[0] : 0.f;
 #pragma unroll 1
@@ -384,9 +387,8 @@ __global__ void __launch_bounds__(256, ConvCfg<BN, NST>::kMaxBlocksPerSm)
               pk[j] = *reinterpret_cast<u32*>(&p2);
             }
             if (inside && a.store) {
-              uint4* dst = reinterpret_cast<uint4*>(o + c0);
-              dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-              dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+              *reinterpret_cast<uint4*>(o + c0 * hw) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+              *reinterpret_cast<uint4*>(o + (c0 + 8) * hw) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
             }
             if (po) {
               u32 mx[8];
@@ -404,9 +406,8 @@ __global__ void __launch_bounds__(256, ConvCfg<BN, NST>::kMaxBlocksPerSm)
                 mx[j] = *reinterpret_cast<u32*>(&r2);
               }
               if (pool_writer) {
-                uint4* dst = reinterpret_cast<uint4*>(po + c0);
-                dst[0] = make_uint4(mx[0], mx[1], mx[2], mx[3]);
-                dst[1] = make_uint4(mx[4], mx[5], mx[6], mx[7]);
+                *reinterpret_cast<uint4*>(po + c0 * (hw >> 2)) = make_uint4(mx[0], mx[1], mx[2], mx[3]);
+                *reinterpret_cast<uint4*>(po + (c0 + 8) * (hw >> 2)) = make_uint4(mx[4], mx[5], mx[6], mx[7]);
               }
             }
             if (a.head_w) {
@@ -458,13 +459,13 @@ struct WgradArgs {
   int* err;
 };
 
-constexpr int kWgPlane = 2944;          // one 18 x 10 x 8-channel halo plane (2880 bytes), 128-byte stride
-constexpr int kWgPlaneBytes = 18 * 10 * 16;
+constexpr int kWgPlane = 18 * 10 * 16;  // one 18 x 10 x 8-channel halo plane (2880 bytes)
 constexpr int kWgDyPlane = 16 * 8 * 16;  // one 16 x 8 x 8-channel dY plane (2048 bytes)
 
 template <int NB, int TAPG, int NST>
 struct WgCfg {
   static constexpr int kSlot = 16 * kWgPlane + (NB / 8) * kWgDyPlane;
+  static_assert(kSlot % 128 == 0 && (16 * kWgPlane) % 128 == 0, "TMA boxes start on 128 bytes");
   static constexpr int kSmem = NST * kSlot + 128 + 1024;  // + barriers, alignment slack
 };
 
@@ -485,7 +486,7 @@ __global__ void __launch_bounds__(128, 1)
   const int t_begin = (int)((int64_t)blockIdx.x * a.tiles / gridDim.x);
   const int t_end = (int)((int64_t)(blockIdx.x + 1) * a.tiles / gridDim.x);
   const int nt = t_end - t_begin;
-  const int planes = min(16, (a.Cx - mb * 128 + 7) / 8);  // halo planes holding real channels (> 0)
+  const int planes = min(16, a.Cx / 8);  // halo planes of a box (past the last channel: zeros)
   const int tx = (a.W + 15) / 16, ty = (a.H + 7) / 8;
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) {
@@ -539,11 +540,9 @@ __global__ void __launch_bounds__(128, 1)
       b -= n * tx * ty;
       const int y0 = (b / tx) * 8, x0 = (b % tx) * 16;
       const u32 hb = sbase + slot * C::kSlot, yb = hb + 16 * kWgPlane;
-      mbar_arrive_tx(full0 + 8 * slot, (u32)(planes * kWgPlaneBytes + (NB / 8) * kWgDyPlane));
-      for (int pl = 0; pl < planes; ++pl)
-        tma_load_4d(hb + pl * kWgPlane, &tmx, mb * 128 + pl * 8, x0 - 1, y0 - 1, n, full0 + 8 * slot);
-      for (int j = 0; j < NB / 8; ++j)
-        tma_load_4d(yb + j * kWgDyPlane, &tmy, nb * NB + j * 8, x0, y0, n, full0 + 8 * slot);
+      mbar_arrive_tx(full0 + 8 * slot, (u32)(planes * kWgPlane + (NB / 8) * kWgDyPlane));
+      tma_load_4d(hb, &tmx, (x0 - 1) * 8, y0 - 1, mb * 16, n, full0 + 8 * slot);
+      tma_load_4d(yb, &tmy, x0 * 8, y0, nb * (NB / 8), n, full0 + 8 * slot);
     }
   }
   // all MMAs of this block done (bounded); then every thread owns TMEM lane tid = input channel
@@ -577,16 +576,16 @@ __global__ void __launch_bounds__(128, 1)
 // decoder input for the weight gradient: [upsampled in0 (c0), in1 (c1)] at full resolution
 __global__ void k_cat_up(const bf16* __restrict__ in0, const bf16* __restrict__ in1, bf16* __restrict__ out, int N,
                          int H, int W, int c0, int c1) {
-  const int cin = c0 + c1, chunks = cin / 8;
-  const int64_t total = (int64_t)N * H * W * chunks;
+  const int chunks = (c0 + c1) / 8, up = c0 / 8;
+  const int64_t hw = (int64_t)H * W, total = (int64_t)N * chunks * hw;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int ch = (int)(i % chunks) * 8;
-    const int64_t p = i / chunks;
-    const int x = (int)(p % W), y = (int)((p / W) % H), n = (int)(p / ((int64_t)W * H));
-    const uint4* src = ch < c0 ? reinterpret_cast<const uint4*>(
-                                     in0 + (((int64_t)n * (H / 2) + y / 2) * (W / 2) + x / 2) * c0 + ch)
-                               : reinterpret_cast<const uint4*>(in1 + p * c1 + (ch - c0));
-    *reinterpret_cast<uint4*>(out + p * cin + ch) = *src;
+    const u32 pl = (u32)i / (u32)hw;  // n * chunks + plane (below 2^32 chunks in all: batches are below 2^27 pixels)
+    const int at = (int)(i - (int64_t)pl * hw), n = (int)(pl / (u32)chunks), ch = (int)(pl - (u32)n * chunks);
+    const int y = at / W, x = at - y * W;
+    const uint4* src = ch < up ? reinterpret_cast<const uint4*>(in0) + ((int64_t)n * up + ch) * (hw >> 2) +
+                                     (int64_t)(y >> 1) * (W >> 1) + (x >> 1)
+                               : reinterpret_cast<const uint4*>(in1) + ((int64_t)n * (chunks - up) + ch - up) * hw + at;
+    reinterpret_cast<uint4*>(out)[i] = *src;
   }
 }
 
@@ -657,44 +656,63 @@ __global__ void k_maxpool_bwd(const bf16* __restrict__ x, const bf16* __restrict
   }
 }
 
-// ReLU gradient in place: dy *= (y > 0), 8 channels (16 bytes) per step
-__global__ void k_relu_bwd(const bf16* __restrict__ y, bf16* __restrict__ dy, int64_t n) {
-  const int64_t n8 = n / 8;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint4 yv = *reinterpret_cast<const uint4*>(y + i * 8);
-    uint4 dv = *reinterpret_cast<const uint4*>(dy + i * 8);
+// ReLU gradient in place, dy *= (y > 0), and the bias gradient db[c] += sum_p dy[p][c] of
+// the result: a block takes a part of one plane of 8 channels of every image (blockIdx.y),
+// 16 bytes per thread and step; the threads' sums meet in shared memory, one atomic per
+// channel and block. One pass over dy instead of two (the sums alone took 15 us a layer).
+__global__ void __launch_bounds__(256) k_relu_bias_bwd(const bf16* __restrict__ y, bf16* __restrict__ dy,
+                                                       float* __restrict__ db, int N, int planes, int64_t hw) {
+  __shared__ float s_db[8];
+  if (threadIdx.x < 8) s_db[threadIdx.x] = 0.f;
+  __syncthreads();
+  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  const int64_t items = (int64_t)N * hw, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += stride) {
+    const int64_t n = (u32)i / (u32)hw, at = (n * planes + blockIdx.y) * hw + (i - n * hw);
+    const uint4 yv = *reinterpret_cast<const uint4*>(y + at * 8);
+    uint4 dv = *reinterpret_cast<const uint4*>(dy + at * 8);
     const __nv_bfloat162* yh = reinterpret_cast<const __nv_bfloat162*>(&yv);
     __nv_bfloat162* dh = reinterpret_cast<__nv_bfloat162*>(&dv);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const float2 f = __bfloat1622float2(yh[j]);
-      const float2 d = __bfloat1622float2(dh[j]);
-      dh[j] = __floats2bfloat162_rn(f.x > 0.f ? d.x : 0.f, f.y > 0.f ? d.y : 0.f);
+      float2 d = __bfloat1622float2(dh[j]);
+      d.x = f.x > 0.f ? d.x : 0.f;
+      d.y = f.y > 0.f ? d.y : 0.f;
+      dh[j] = __floats2bfloat162_rn(d.x, d.y);
+      acc[2 * j] += d.x;
+      acc[2 * j + 1] += d.y;
     }
-    *reinterpret_cast<uint4*>(dy + i * 8) = dv;
+    *reinterpret_cast<uint4*>(dy + at * 8) = dv;
   }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s_db[j], acc[j]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 8) atomicAdd(&db[blockIdx.y * 8 + threadIdx.x], s_db[threadIdx.x]);
 }
 
 // gradient of concat([upsample(low), skip]): low gets the 2x2 sums of the
 // first c_up channels, skip the remaining channels; 8 channels (16 bytes) per step
 __global__ void k_split_cat_bwd(const bf16* __restrict__ dcat, bf16* __restrict__ dlow,
                                 bf16* __restrict__ dskip, int N, int H, int W, int c_up, int c_skip) {
-  const int Ho = H / 2, Wo = W / 2;
-  const int C = c_up + c_skip, cu8 = c_up / 8, cs8 = c_skip / 8;
-  const int64_t tl = (int64_t)N * Ho * Wo * cu8;
+  const int Wo = W / 2;
+  const int cu8 = c_up / 8, cs8 = c_skip / 8, c8 = cu8 + cs8;
+  const int64_t hw = (int64_t)H * W, hwo = hw >> 2;
+  const int64_t tl = (int64_t)N * cu8 * hwo;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < tl; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i % cu8) * 8;
-    int64_t r = i / cu8;
-    const int xo = (int)(r % Wo);
-    r /= Wo;
-    const int yo = (int)(r % Ho);
-    const int n = (int)(r / Ho);
-    const int64_t b = (((int64_t)n * H + 2 * yo) * W + 2 * xo) * C + c;
-    const int64_t off[4] = {0, C, (int64_t)W * C, (int64_t)W * C + C};
+    const u32 pl = (u32)i / (u32)hwo;  // n * cu8 + plane
+    const int at = (int)(i - (int64_t)pl * hwo), n = (int)(pl / (u32)cu8), c = (int)(pl - (u32)n * cu8);
+    const int yo = at / Wo, xo = at - yo * Wo;
+    const bf16* b = dcat + (((int64_t)n * c8 + c) * hw + (int64_t)(2 * yo) * W + 2 * xo) * 8;
+    const int64_t off[4] = {0, 8, (int64_t)W * 8, (int64_t)W * 8 + 8};
     float s[8];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const uint4 v = *reinterpret_cast<const uint4*>(dcat + b + off[k]);
+      const uint4 v = *reinterpret_cast<const uint4*>(b + off[k]);
       const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -709,42 +727,12 @@ __global__ void k_split_cat_bwd(const bf16* __restrict__ dcat, bf16* __restrict_
     for (int j = 0; j < 4; ++j) oh[j] = __floats2bfloat162_rn(s[2 * j], s[2 * j + 1]);
     *reinterpret_cast<uint4*>(dlow + i * 8) = o;
   }
-  const int64_t ts = (int64_t)N * H * W * cs8;
+  const int64_t ts = (int64_t)N * cs8 * hw;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ts; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i % cs8) * 8;
-    const int64_t p = i / cs8;
-    *reinterpret_cast<uint4*>(dskip + i * 8) = *reinterpret_cast<const uint4*>(dcat + p * C + c_up + c);
+    const u32 pl = (u32)i / (u32)hw, n = pl / (u32)cs8, c = pl - n * cs8;
+    *reinterpret_cast<uint4*>(dskip + i * 8) =
+        *reinterpret_cast<const uint4*>(dcat + (((int64_t)n * c8 + cu8 + c) * hw + (i - (int64_t)pl * hw)) * 8);
   }
-}
-
-// bias gradient: db[c] += sum over pixels of dy[p][c]
-// bias gradient db[c] += sum_p dy[p][c]: a thread owns one 8-channel chunk (16-byte loads) over
-// a stride of pixels; partial sums meet in shared memory, one atomic per channel per block
-__global__ void k_bias_grad(const bf16* __restrict__ dy, float* __restrict__ db, int64_t P, int C) {
-  __shared__ float s_db[256];
-  for (int c = threadIdx.x; c < C; c += blockDim.x) s_db[c] = 0.f;
-  __syncthreads();
-  const int chunks = C / 8;  // divides the grid's thread count, so a thread keeps its chunk
-  const int64_t items = P * chunks, stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  for (int64_t i = i0; i < items; i += stride) {
-    const uint4 v = *reinterpret_cast<const uint4*>(dy + i * 8);
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 f = __bfloat1622float2(h[j]);
-      acc[2 * j] += f.x;
-      acc[2 * j + 1] += f.y;
-    }
-  }
-  if (i0 < items) {
-    const int k = (int)(i0 % chunks) * 8;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) atomicAdd(&s_db[k + j], acc[j]);
-  }
-  __syncthreads();
-  for (int c = threadIdx.x; c < C; c += blockDim.x) atomicAdd(&db[c], s_db[c]);
 }
 
 __device__ __forceinline__ float warp_sum(float x) {
@@ -759,7 +747,7 @@ __device__ __forceinline__ float warp_sum(float x) {
 // (one shared-memory add per warp and channel), skipped where no lane has a hidden cell.
 __global__ void k_head(const bf16* __restrict__ d1, int C, const float* __restrict__ w, const float* __restrict__ b,
                        const float* __restrict__ fill, float* __restrict__ pred, const float* __restrict__ target,
-                       const uint8_t* __restrict__ hidden, float inv_cnt, int64_t P, float* __restrict__ loss,
+                       const uint8_t* __restrict__ hidden, float inv_cnt, int64_t P, int64_t hw, float* __restrict__ loss,
                        bf16* __restrict__ dd1, float* __restrict__ dw, float* __restrict__ dbias) {
   __shared__ float s_w[256], s_dw[256];
   __shared__ float s_loss, s_db;
@@ -776,11 +764,13 @@ __global__ void k_head(const bf16* __restrict__ d1, int C, const float* __restri
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < P; base += stride) {
     const int64_t p = base + threadIdx.x;
     const bool in = p < P;
+    // channel c (a multiple of 8) of the pixel is at c hw + d0
+    const int64_t n = in ? (u32)p / (u32)hw : 0, d0 = n * hw * C + (in ? p - n * hw : 0) * 8;
     float g = 0.f;
     if (in) {
       float r = b[0];
       for (int c = 0; c < C; c += 8) {
-        const uint4 v = *reinterpret_cast<const uint4*>(d1 + p * C + c);
+        const uint4 v = *reinterpret_cast<const uint4*>(d1 + d0 + c * hw);
         const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -803,14 +793,14 @@ __global__ void k_head(const bf16* __restrict__ d1, int C, const float* __restri
             __nv_bfloat162 q = __floats2bfloat162_rn(g * s_w[c + 2 * j], g * s_w[c + 2 * j + 1]);
             o[j] = *reinterpret_cast<u32*>(&q);
           }
-          *reinterpret_cast<uint4*>(dd1 + p * C + c) = make_uint4(o[0], o[1], o[2], o[3]);
+          *reinterpret_cast<uint4*>(dd1 + d0 + c * hw) = make_uint4(o[0], o[1], o[2], o[3]);
         }
       }
     }
     if (target && __any_sync(0xffffffffu, g != 0.f)) {
       for (int c = 0; c < C; c += 8) {
         uint4 v = make_uint4(0, 0, 0, 0);
-        if (in) v = *reinterpret_cast<const uint4*>(d1 + p * C + c);
+        if (in) v = *reinterpret_cast<const uint4*>(d1 + d0 + c * hw);
         const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -1040,14 +1030,15 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
-// NHWC bf16 activations [n][h][w][c] as a 4-D tensor (c innermost) read in boxes of
-// 8 channels x box x box pixels; false if the encoder is unavailable or refuses
-bool activation_map(CUtensorMap* m, const bf16* base, int c, int w, int h, int n, int box) {
+// Activations [n][c / 8][h][w][8] as a 4-D tensor (8 w values of a row, rows, planes, images)
+// read in boxes of bw x bh pixels of `planes` planes; false if the encoder is unavailable or
+// refuses. A box starts at a multiple of 8 values, 16 bytes.
+bool activation_map(CUtensorMap* m, const bf16* base, int c, int w, int h, int n, int bw, int bh, int planes) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  if (!enc) return false;
-  const cuuint64_t dims[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
-  const cuuint64_t strides[3] = {(cuuint64_t)c * 2, (cuuint64_t)c * 2 * w, (cuuint64_t)c * 2 * w * h};
-  const cuuint32_t boxd[4] = {8, (cuuint32_t)box, (cuuint32_t)box, 1};
+  if (!enc || c % 8) return false;
+  const cuuint64_t dims[4] = {(cuuint64_t)w * 8, (cuuint64_t)h, (cuuint64_t)c / 8, (cuuint64_t)n};
+  const cuuint64_t strides[3] = {(cuuint64_t)w * 16, (cuuint64_t)w * 16 * h, (cuuint64_t)c * 2 * w * h};
+  const cuuint32_t boxd[4] = {(cuuint32_t)bw * 8, (cuuint32_t)bh, (cuuint32_t)planes, 1};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(base), dims, strides, boxd, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -1099,10 +1090,11 @@ cudaError_t conv(mem_unet* u, const ConvLayer& c, const bf16* in0, const bf16* i
     return cudaErrorInvalidValue;
   CUtensorMap tm0, tm1;
   // (c_stored: channels that in0 holds where fewer than c0; the loads of the others read zero)
-  if (!activation_map(&tm0, in0, c_stored ? c_stored : c0, up0 ? W / 2 : W, up0 ? H / 2 : H, N, up0 ? kHalfBox : kHX))
+  if (!activation_map(&tm0, in0, c_stored ? c_stored : c0, up0 ? W / 2 : W, up0 ? H / 2 : H, N, up0 ? kHalfBox : kHX,
+                      up0 ? kHalfBox : kHY, 2))
     return cudaErrorInvalidValue;
   if (c1) {
-    if (!activation_map(&tm1, in1, c1, W, H, N, kHX)) return cudaErrorInvalidValue;
+    if (!activation_map(&tm1, in1, c1, W, H, N, kHX, kHY, 2)) return cudaErrorInvalidValue;
   } else {
     tm1 = tm0;
   }
@@ -1130,19 +1122,6 @@ void launch_wgrad(dim3 grid, const CUtensorMap& tmx, const CUtensorMap& tmy, con
   k_wgrad3x3t<NB, TAPG, NST><<<grid, 128, C::kSmem, st>>>(tmx, tmy, a);
 }
 
-// NHWC bf16 tensor [n][h][w][c] as a 4-D tensor map with boxes of 8 channels x bw x bh pixels
-bool nhwc_map(CUtensorMap* m, const bf16* base, int c, int w, int h, int n, int bw, int bh) {
-  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  if (!enc) return false;
-  const cuuint64_t dims[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
-  const cuuint64_t strides[3] = {(cuuint64_t)c * 2, (cuuint64_t)c * 2 * w, (cuuint64_t)c * 2 * w * h};
-  const cuuint32_t boxd[4] = {8, (cuuint32_t)bw, (cuuint32_t)bh, 1};
-  const cuuint32_t estr[4] = {1, 1, 1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(base), dims, strides, boxd, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // dW (float32, [9][cin_pad][cout], accumulated into) of one 3x3 convolution whose input is
 // in0 (c0 channels; at half resolution when up0) concatenated with in1 (c1 channels)
 cudaError_t wgrad(mem_unet* u, const ConvLayer& c, const bf16* in0, const bf16* in1, const bf16* dy,
@@ -1156,9 +1135,6 @@ cudaError_t wgrad(mem_unet* u, const ConvLayer& c, const bf16* in0, const bf16* 
     X = u->dcat;
   }
   if (Cx % 8 || c.cout % 32 || c.cin_pad % 8 || Cx > c.cin_pad) return cudaErrorInvalidValue;
-  CUtensorMap tmx, tmy;
-  if (!nhwc_map(&tmx, X, Cx, W, H, N, 18, 10) || !nhwc_map(&tmy, dy, c.cout, W, H, N, 16, 8))
-    return cudaErrorInvalidValue;
   WgradArgs a;
   a.Cx = Cx;
   a.cin_pad = c.cin_pad;
@@ -1172,6 +1148,10 @@ cudaError_t wgrad(mem_unet* u, const ConvLayer& c, const bf16* in0, const bf16* 
   // output-channel block and tap group: TMEM holds the tap group's accumulators (<= 512 columns)
   const int NB = c.cout % 128 == 0 ? 128 : (c.cout % 64 == 0 ? 64 : 32);
   const int TAPG = NB == 128 ? 3 : (NB == 64 ? 5 : 9);
+  CUtensorMap tmx, tmy;
+  if (!activation_map(&tmx, X, Cx, W, H, N, 18, 10, Cx / 8 < 16 ? Cx / 8 : 16) ||
+      !activation_map(&tmy, dy, c.cout, W, H, N, 16, 8, NB / 8))
+    return cudaErrorInvalidValue;
   const int mbk = (Cx + 127) / 128, groups = (c.cout / NB) * ((9 + TAPG - 1) / TAPG);
   int splits = (u->n_sm + mbk * groups - 1) / (mbk * groups);  // about one block per SM
   if (splits > a.tiles / 8) splits = a.tiles / 8;  // at least 8 tiles per block: the epilogue's atomics
@@ -1253,7 +1233,12 @@ cudaError_t backward(mem_unet* u, int N, int H, int W, cudaStream_t st) {
     const int l = c.level;
     const int Hl = H >> l, Wl = W >> l;
     const int64_t Pl = (int64_t)N * Hl * Wl;
-    k_relu_bwd<<<grid_for(Pl * c.cout / 8, u->n_sm), 256, 0, st>>>(u->act[i], u->dact[i], Pl * c.cout);
+    {
+      const int planes = c.cout / 8;
+      const int parts = std::max(1, std::min((u->n_sm * 8 + planes - 1) / planes, (int)std::min<int64_t>((Pl + 255) / 256, 1 << 20)));
+      k_relu_bias_bwd<<<dim3(parts, planes), 256, 0, st>>>(u->act[i], u->dact[i], u->grads + c.b_off, N, planes,
+                                                           (int64_t)Hl * Wl);
+    }
     ConvLayer cc = c;
     if (i == 0) cc.c0 = kInC;
     float* dw = i == 0 ? u->g0pad : u->grads + c.w_off;  // only the first layer has padded rows
@@ -1263,8 +1248,6 @@ cudaError_t backward(mem_unet* u, int N, int H, int W, cudaStream_t st) {
     if (i == 0)
       k_unpad_rows<<<grid_for(9LL * c.cin * c.cout, u->n_sm), 256, 0, st>>>(u->g0pad, u->grads + c.w_off, c.cin,
                                                                             c.cin_pad, c.cout);
-    // bias gradient
-    k_bias_grad<<<u->n_sm * 2, 256, 0, st>>>(u->dact[i], u->grads + c.b_off, Pl, c.cout);
     if (i == 0) break;
     // data gradient into the layer input
     if (c.c1) {  // decoder concat input: d(concat) then split
@@ -1283,7 +1266,7 @@ cudaError_t backward(mem_unet* u, int N, int H, int W, cudaStream_t st) {
       const int src = i - 1;
       const ConvLayer& ps = u->L[src];
       k_maxpool_bwd<<<grid_for((int64_t)N * Hl * Wl * ps.cout / 8, u->n_sm), 256, 0, st>>>(
-          u->act[src], u->dpool[lv], u->dact[src], N, Hl * 2, Wl * 2, ps.cout);
+          u->act[src], u->dpool[lv], u->dact[src], N * (ps.cout / 8), Hl * 2, Wl * 2, 8);  // planes as images
     } else {
       e = conv(u, c, u->dact[i], nullptr, c.wd, nullptr, u->dact[i - 1], c.cin, c.cout_pad, c.cout, 0, 0, N, Hl, Wl,
                0, st);
@@ -1437,7 +1420,7 @@ extern "C" mem_status mem_unet_forward(mem_unet* u, int32_t n, int32_t H, int32_
   if (!head_done)
     k_head<<<grid_for(P, u->n_sm), 256, 0, st>>>(u->act[13], u->widths[0], u->params + u->head_w,
                                                   u->params + u->head_b, fill, pred, nullptr, nullptr, 0.f, P,
-                                                  nullptr, nullptr, nullptr, nullptr);
+                                                  (int64_t)H * W, nullptr, nullptr, nullptr, nullptr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return memh::api_cuda_fail(e, "U-Net head");
   return MEM_OK;
@@ -1468,7 +1451,7 @@ extern "C" mem_status mem_unet_gradients(mem_unet* u, int32_t n, int32_t H, int3
   const float inv = 1.f / (float)(n_hidden > 0 ? n_hidden : 1);
   k_head<<<grid_for(P, u->n_sm), 256, 0, st>>>(u->act[13], u->widths[0], u->params + u->head_w,
                                                 u->params + u->head_b, fill, nullptr, target, hidden, inv, P,
-                                                u->d_loss, u->dact[13], u->grads + u->head_w, u->grads + u->head_b);
+                                                (int64_t)H * W, u->d_loss, u->dact[13], u->grads + u->head_w, u->grads + u->head_b);
   e = backward(u, n, H, W, st);
   if (e != cudaSuccess) return memh::api_cuda_fail(e, "U-Net backward");
   if (grads) e = cudaMemcpyAsync(grads, u->grads, u->n_params * 4, cudaMemcpyDeviceToDevice, st);
