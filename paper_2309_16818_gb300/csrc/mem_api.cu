@@ -388,13 +388,18 @@ static void camera_rel(const double T[16], const double o[2], MapCall& mc) {
   mc.cam_h = (float)d[2];
 }
 
-// Stage a job block in a pinned slot and queue its copy to the device.
-static mem_status stage_job(Map* m, int jb, const void* host, size_t bytes, cudaStream_t st) {
-  if (bytes > m->job_bytes) return fail(MEM_ERR_STATE, "job block too large (%zu bytes)", bytes);
+// The next pinned slot for a job block, free to be written.
+static mem_status job_slot(Map* m, int* slot) {
   const int s = m->job_slot;
   m->job_slot = (s + 1) % kJobSlots;
   CK(cudaEventSynchronize(m->job_ev[s]), "cudaEventSynchronize");
-  memcpy(m->h_job[s], host, bytes);
+  *slot = s;
+  return MEM_OK;
+}
+
+// Queue the copy of a job block built in pinned slot `s` to device block `jb`.
+static mem_status stage_job(Map* m, int jb, int s, size_t bytes, cudaStream_t st) {
+  if (bytes > m->job_bytes) return fail(MEM_ERR_STATE, "job block too large (%zu bytes)", bytes);
   CK(cudaMemcpyAsync(m->d_job[jb], m->h_job[s], bytes, cudaMemcpyHostToDevice, st), "job upload");
   CK(cudaEventRecord(m->job_ev[s], st), "cudaEventRecord");
   return MEM_OK;
@@ -679,7 +684,7 @@ static mem_status check_sources(const Map* m, int32_t n_sources, const mem_sourc
 // The warp fuse kernel's plan (n_rounds 0 when the call exceeds its tables).
 static void build_plan(memk::FusePlan& p, const PointJob& job, const LayerDev* L) {
   using memk::kFuseQ;
-  memset(&p, 0, sizeof(p));
+  memset(&p, 0, offsetof(memk::FusePlan, seg));  // the tables after it are written as far as they are used
   int r = 0, col = 4, ns = 0, nt = 0;
   for (int c = 0; c < 4; ++c) p.slot[c] = (unsigned short)c;
   auto close = [&]() {  // the round is full (or the call ends)
@@ -849,8 +854,10 @@ static mem_status run_points(Map* m, int nm, const int64_t* offsets, int64_t n, 
                              cudaStream_t job_st = nullptr, cudaEvent_t ready = nullptr, int jb = kJobDevice) {
   mem_status s = ensure_capacity(m, n);
   if (s != MEM_OK) return s;
-  std::string buf(m->job_bytes, '\0');
-  char* h = &buf[0];
+  int slot = 0;  // the block is built in the pinned memory it is copied from
+  s = job_slot(m, &slot);
+  if (s != MEM_OK) return s;
+  char* h = m->h_job[slot];
   PointJob* job = (PointJob*)h;
   // [job][plan][map calls][offsets]
   constexpr size_t plan_at = (sizeof(PointJob) + 15) & ~(size_t)15, maps_at = plan_at + sizeof(memk::FusePlan);
@@ -900,7 +907,7 @@ static mem_status run_points(Map* m, int nm, const int64_t* offsets, int64_t n, 
     for (int b = 0; b <= nm; ++b) offs[b] = offsets[b];
     bytes = offs_at + sizeof(int64_t) * (nm + 1);
   }
-  s = stage_job(m, jb, h, bytes, ready ? job_st : st);
+  s = stage_job(m, jb, slot, bytes, ready ? job_st : st);
   if (s != MEM_OK) return s;
   if (ready) {
     CK(cudaEventRecord(ready, job_st), "job upload record");

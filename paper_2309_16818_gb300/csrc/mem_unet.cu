@@ -573,13 +573,19 @@ __global__ void __launch_bounds__(128, 1)
   }
 }
 
+// i / d for i < total; in 32 bits wherever the total allows (a 64-bit division costs more than
+// the 16-byte copy it is for)
+__device__ __forceinline__ u32 div_i(int64_t i, int64_t d, int64_t total) {
+  return total >> 32 ? (u32)(i / d) : (u32)i / (u32)d;
+}
+
 // decoder input for the weight gradient: [upsampled in0 (c0), in1 (c1)] at full resolution
 __global__ void k_cat_up(const bf16* __restrict__ in0, const bf16* __restrict__ in1, bf16* __restrict__ out, int N,
                          int H, int W, int c0, int c1) {
   const int chunks = (c0 + c1) / 8, up = c0 / 8;
   const int64_t hw = (int64_t)H * W, total = (int64_t)N * chunks * hw;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const u32 pl = (u32)i / (u32)hw;  // n * chunks + plane (below 2^32 chunks in all: batches are below 2^27 pixels)
+    const u32 pl = div_i(i, hw, total);  // n * chunks + plane
     const int at = (int)(i - (int64_t)pl * hw), n = (int)(pl / (u32)chunks), ch = (int)(pl - (u32)n * chunks);
     const int y = at / W, x = at - y * W;
     const uint4* src = ch < up ? reinterpret_cast<const uint4*>(in0) + ((int64_t)n * up + ch) * (hw >> 2) +
@@ -704,7 +710,7 @@ __global__ void k_split_cat_bwd(const bf16* __restrict__ dcat, bf16* __restrict_
   const int64_t hw = (int64_t)H * W, hwo = hw >> 2;
   const int64_t tl = (int64_t)N * cu8 * hwo;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < tl; i += (int64_t)gridDim.x * blockDim.x) {
-    const u32 pl = (u32)i / (u32)hwo;  // n * cu8 + plane
+    const u32 pl = div_i(i, hwo, tl);  // n * cu8 + plane
     const int at = (int)(i - (int64_t)pl * hwo), n = (int)(pl / (u32)cu8), c = (int)(pl - (u32)n * cu8);
     const int yo = at / Wo, xo = at - yo * Wo;
     const bf16* b = dcat + (((int64_t)n * c8 + c) * hw + (int64_t)(2 * yo) * W + 2 * xo) * 8;
@@ -729,7 +735,7 @@ __global__ void k_split_cat_bwd(const bf16* __restrict__ dcat, bf16* __restrict_
   }
   const int64_t ts = (int64_t)N * cs8 * hw;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ts; i += (int64_t)gridDim.x * blockDim.x) {
-    const u32 pl = (u32)i / (u32)hw, n = pl / (u32)cs8, c = pl - n * cs8;
+    const u32 pl = div_i(i, hw, ts), n = pl / (u32)cs8, c = pl - n * cs8;
     *reinterpret_cast<uint4*>(dskip + i * 8) =
         *reinterpret_cast<const uint4*>(dcat + (((int64_t)n * c8 + cu8 + c) * hw + (i - (int64_t)pl * hw)) * 8);
   }
