@@ -358,7 +358,8 @@ __global__ void __launch_bounds__(256) k_pca_cov_final(PcaArgs a, int nt, int ti
 // barriers a step; the pairs of step t are computed from t; a warp per row of
 // blocks, so no divisions). Bound by the latency of its steps; with the sides one
 // after the other, V with them and the round-robin order moved along by one
-// thread (four barriers a step) 64 channels took 609 us, now 314 us.
+// thread (four barriers a step) 64 channels took 609 us, now 314 us and 34 us for
+// the corrections of three vectors (5e-8 from the float64 vectors, 3e-6 to 1e-5 without).
 // the angles of step `step`: round-robin, position 0 holds row 0, position i >= 1 row
 // 1 + (i - 1 - step) mod (n - 1); pair m: positions m and n - 1 - m. By one warp.
 __device__ __forceinline__ void jacobi_angles(const float* A, int ld, int n, int step, float4* rot) {
@@ -384,6 +385,97 @@ __device__ __forceinline__ void jacobi_angles(const float* A, int ld, int n, int
   }
 }
 
+__device__ __forceinline__ double warp_sum_d(double x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// Kept eigenvector k (column `sel` of V) by the whole block: the rotations leave it with
+// float32 rounding of several hundred steps, a few 1e-6; one first-order correction with the
+// covariance itself (its product with v in float64), v += sum_j (u_j . r) / (lambda - lambda_j) u_j with the
+// residual r = A v - lambda v, squares that error. Directions whose eigenvalue is as good as
+// equal (a coefficient of 1 % or more) are left alone. Then normalised, signed by its
+// largest-magnitude component (the smaller index first on ties) and written, with its
+// Rayleigh quotient as the eigenvalue.
+__device__ void refine_vector(const float* A, const float* V, int ld, int n, const PcaArgs& a, int sel, int k) {
+  __shared__ double s_v[kPcaMaxC], s_r[kPcaMaxC], s_lam, s_scale;
+  __shared__ float s_f[kPcaMaxC], s_c[kPcaMaxC];  // the residual and the coefficients: float32 carries a correction
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, C = a.C;
+  for (int i = threadIdx.x; i < C; i += blockDim.x) s_v[i] = (double)V[i * ld + sel];
+  __syncthreads();
+  for (int i = warp; i < C; i += 32) {  // A v
+    double y = 0.0;
+    for (int j = lane; j < C; j += 32) y = fma((double)a.cov[i * C + j], s_v[j], y);
+    y = warp_sum_d(y);
+    if (lane == 0) s_r[i] = y;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    double vy = 0.0, vv = 0.0;
+    for (int i = lane; i < C; i += 32) {
+      vy = fma(s_v[i], s_r[i], vy);
+      vv = fma(s_v[i], s_v[i], vv);
+    }
+    vy = warp_sum_d(vy);
+    vv = warp_sum_d(vv);
+    if (lane == 0) s_lam = vv > 0.0 ? vy / vv : 0.0;
+  }
+  __syncthreads();
+  const double lam = s_lam;
+  for (int i = threadIdx.x; i < C; i += blockDim.x) s_f[i] = (float)(s_r[i] - lam * s_v[i]);
+  __syncthreads();
+  for (int j = warp; j < n; j += 32) {  // u_j . r
+    float d = 0.f;
+    for (int i = lane; i < C; i += 32) d = fmaf(V[i * ld + j], s_f[i], d);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if (lane == 0) {
+      const float gap = (float)lam - A[j * (ld + 1)];
+      s_c[j] = j != sel && fabsf(d) < 0.01f * fabsf(gap) ? d / gap : 0.f;
+    }
+  }
+  __syncthreads();
+  for (int i = warp; i < C; i += 32) {
+    float x = 0.f;
+    for (int j = lane; j < n; j += 32) x = fmaf(s_c[j], V[i * ld + j], x);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (lane == 0) s_r[i] = s_v[i] + (double)x;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    double vv = 0.0, mv = -1.0;
+    int mi = C;
+    for (int i = lane; i < C; i += 32) {
+      vv = fma(s_r[i], s_r[i], vv);
+      const double v = (double)(float)fabs(s_r[i]);
+      if (v > mv) {
+        mv = v;
+        mi = i;
+      }
+    }
+    vv = warp_sum_d(vv);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ov = __shfl_xor_sync(0xffffffffu, mv, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
+      if (ov > mv || (ov == mv && oi < mi)) {
+        mv = ov;
+        mi = oi;
+      }
+    }
+    if (lane == 0) {
+      const double inv = vv > 0.0 ? 1.0 / sqrt(vv) : 1.0;
+      s_scale = mi < C && s_r[mi] < 0.0 ? -inv : inv;
+      a.vals[k] = (float)lam;
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < C; i += blockDim.x) a.vecs[k * C + i] = (float)(s_r[i] * s_scale);
+  __syncthreads();
+}
+
 __global__ void __launch_bounds__(1024) k_pca_eig(PcaArgs a) {
   extern __shared__ float sm[];
   const int C = a.C, n = (C + 1) & ~1;
@@ -400,6 +492,7 @@ __global__ void __launch_bounds__(1024) k_pca_eig(PcaArgs a) {
   }
   __syncthreads();
   __shared__ float red[2][32];
+  __shared__ int s_sel[kPcaMaxComp];
   // converged when the off-diagonal mass is at the float32 rounding level of the matrix
   const float conv = (4.f * n * 5.96e-8f) * (4.f * n * 5.96e-8f);
   for (int sweep = 0; sweep < 20; ++sweep) {
@@ -469,8 +562,7 @@ __global__ void __launch_bounds__(1024) k_pca_eig(PcaArgs a) {
       __syncthreads();
     }
   }
-  // the n_comp largest eigenvalues (the smaller index first on ties), each vector signed by its
-  // largest-magnitude component (the smaller index first on ties), by one warp
+  // the n_comp largest eigenvalues (the smaller index first on ties), by one warp
   if (warp == 0) {
     u32 taken = 0;  // bit j: diagonal entry lane + 32 j is used
     for (int k = 0; k < a.n_comp; ++k) {
@@ -493,29 +585,14 @@ __global__ void __launch_bounds__(1024) k_pca_eig(PcaArgs a) {
         }
       }
       if ((bi & 31) == lane) taken |= 1u << (bi >> 5);
-      float mv = -1.f;
-      int mi = n;
-      for (int r = lane; r < C; r += 32) {
-        const float v = fabsf(V[r * ld + bi]);
-        if (v > mv) {
-          mv = v;
-          mi = r;
-        }
+      if (lane == 0) {
+        s_sel[k] = bi;
+        a.vals[k] = bv;
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, mv, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
-        if (ov > mv || (ov == mv && oi < mi)) {
-          mv = ov;
-          mi = oi;
-        }
-      }
-      const float sg = mi < n && V[mi * ld + bi] < 0.f ? -1.f : 1.f;
-      if (lane == 0) a.vals[k] = bv;
-      for (int r = lane; r < C; r += 32) a.vecs[k * C + r] = sg * V[r * ld + bi];
     }
   }
+  __syncthreads();
+  for (int k = 0; k < a.n_comp; ++k) refine_vector(A, V, ld, n, a, s_sel[k], k);
   __syncthreads();
   if (a.info) {
     for (int k = threadIdx.x; k < a.n_comp; k += blockDim.x) a.info[k] = a.vals[k];
