@@ -251,6 +251,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(MapDev md, const P
   const int64_t n = job->n;
   const int n_tiles = (int)((n + kTile - 1) / kTile);
   const int shift = pass * RB;
+  // (plain loads: the keys and indices are the previous kernel's, see pdl_wait; they also measured faster
+  // than read-only or L2-only ones, 16.0 against 17.0 us a pass of 569k points)
   const u32* kin = (pass & 1) ? md.keys1 : md.keys0;
   u32* __restrict__ kout = (pass & 1) ? md.keys0 : md.keys1;
   const u32* vin = (pass & 1) ? md.vals1 : md.vals0;
@@ -297,8 +299,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(MapDev md, const P
     for (int j = 0; j < kSortItems; ++j) {
       const int64_t idx = wbase + j * 32 + lane;
       const bool ok = idx < n;
-      key[j] = ok ? __ldcg(kin + idx) : 0xffffffffu;
-      val[j] = ok ? (pass == 0 ? (u32)idx : __ldcg(vin + idx)) : 0u;
+      key[j] = ok ? kin[idx] : 0xffffffffu;
+      val[j] = ok ? (pass == 0 ? (u32)idx : vin[idx]) : 0u;
     }
     // ranks within the warp, in (item, lane) order = input order
 #pragma unroll
@@ -908,11 +910,11 @@ __global__ void __launch_bounds__(kFT, 7) k_fuse_tiles(MapDev md, const PointJob
     const int np = (int)min((int64_t)kFT, n_kept - p0);
     // A. keys, point indices, runs
     if (t < np) {
-      s.key[t + 1] = __ldcg(sk + p0 + t);
-      s.idx[t] = __ldcg(sv + p0 + t);
+      s.key[t + 1] = sk[p0 + t];
+      s.idx[t] = sv[p0 + t];
     }
-    if (t == 0) s.key[0] = p0 > 0 ? __ldcg(sk + p0 - 1) : 0xfffffffeu;
-    if (t == 32) s.key[np + 1] = (p0 + np < n_kept) ? __ldcg(sk + p0 + np) : 0xfffffffeu;
+    if (t == 0) s.key[0] = p0 > 0 ? sk[p0 - 1] : 0xfffffffeu;
+    if (t == 32) s.key[np + 1] = (p0 + np < n_kept) ? sk[p0 + np] : 0xfffffffeu;
     __syncthreads();
     const bool hd = t < np && (t == 0 || s.key[t] != s.key[t + 1]);
     const bool ed = t < np && (t == np - 1 || s.key[t + 1] != s.key[t + 2]);
@@ -1650,10 +1652,10 @@ __global__ void __launch_bounds__(kFT, kWarpBlocks) k_fuse_warps(MapDev md, cons
     // A. key, neighbours' keys, runs and pieces
     u32 key = 0xfffffffeu, kprev = 0xfffffffeu, knext = 0xfffffffeu, id = 0;
     if (on) {
-      key = __ldcg(sk + p);
-      id = __ldcg(sv + p);
-      if (p > 0) kprev = __ldcg(sk + p - 1);
-      if (p + 1 < n_kept) knext = __ldcg(sk + p + 1);
+      key = sk[p];
+      id = sv[p];
+      if (p > 0) kprev = sk[p - 1];
+      if (p + 1 < n_kept) knext = sk[p + 1];
     }
     __syncthreads();  // plan in place; the previous tile is done with the shared arrays
     const bool hd = on && key != kprev;  // a run begins here
