@@ -406,7 +406,8 @@ mem_status mem_unet_forward(mem_unet *u, int32_t n, int32_t H, int32_t W, const 
                             const float *fill, float *pred, void *stream);
 /* loss = sum over hidden cells of (pred - target)^2 / n_hidden (device
  * float32, optional) and its gradient for every parameter into grads (flat,
- * optional) */
+ * optional). Sums are taken in a fixed order: the same parameters and batch give
+ * the same bits. */
 mem_status mem_unet_gradients(mem_unet *u, int32_t n, int32_t H, int32_t W, const float *x3,
                               const float *fill, const float *target, const uint8_t *hidden,
                               int64_t n_hidden, float *grads, float *loss, void *stream);

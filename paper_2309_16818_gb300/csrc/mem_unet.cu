@@ -16,7 +16,14 @@
 // half-resolution box replicated in shared memory. The data gradient is the
 // same kernel with flipped, transposed weights; the weight gradient is a
 // tcgen05 GEMM over pixels (both operands MN-major from TMA-loaded planes, one
-// TMEM accumulator per tap) split across blocks with float32 atomics.
+// TMEM accumulator per tap) split across blocks.
+//
+// Every sum of the backward pass is taken in a fixed order: blocks leave partial sums in a
+// scratch buffer and k_grad_sum adds them, so that the same state and batch give the same
+// gradients bit for bit. With float32 atomics the order, and 1e-7 to 4e-7 of a gradient, was
+// another one in every call; Adam divides by the gradient's own size, so weights with gradients
+// of 1e-8 and less moved visibly by it (parameters after two steps on 16 crops of 256 x 256:
+// up to 5e-5 of their norm between two runs of the same program).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <math.h>
@@ -447,13 +454,13 @@ __global__ void __launch_bounds__(256, ConvCfg<BN, NST>::kMaxBlocksPerSm)
 // ((py + dy) * 18 + dx) pixels, 128 bytes between the two 8-pixel halves of K
 // and one plane between 8-channel groups of M (and N). Each tap of the block's
 // tap group accumulates in its own TMEM columns over all tiles of the block's
-// pixel range; the epilogue adds the float32 sums to dW with atomics (blocks
-// split the pixels). Warp 0: TMEM and the MMA thread; warp 1: one thread
+// pixel range; the epilogue stores the float32 sums as the block's part of dW (blocks
+// split the pixels; k_grad_sum adds the parts). Warp 0: TMEM and the MMA thread; warp 1: one thread
 // issues the copies; all four warps drain TMEM at the end. Waits are bounded.
 
 struct WgradArgs {
-  int Cx, cin_pad, cout;  // input channels in the tensor (real), rows of dW per tap, dY channels
-  float* dw;              // [9][cin_pad][cout] float32, accumulated into
+  int Cx, cout;           // input channels in the tensor, dY channels
+  float* part;            // [gridDim.x][9][Cx][cout] float32
   int N, H, W;
   int tiles;              // 16 x 8 pixel tiles over the batch
   int* err;
@@ -550,18 +557,18 @@ __global__ void __launch_bounds__(128, 1)
   tc_fence_after();
   ok = __all_sync(0xffffffffu, ok) && nt > 0;
   const int ci = mb * 128 + tid;
-  if (ok) {
-    for (int tl = 0; tl < n_taps; ++tl) {
-      const int t = t_first + tl;
+  for (int tl = 0; tl < n_taps; ++tl) {
+    const int t = t_first + tl;
 #pragma unroll 1
-      for (int c0 = 0; c0 < NB; c0 += 16) {
-        u32 v[16];
-        tmem_ld16(tmem + ((u32)(warp * 32) << 16) + (u32)(tl * NB + c0), v);
-        if (ci < a.Cx && ci < a.cin_pad) {
-          float* d = a.dw + ((int64_t)t * a.cin_pad + ci) * a.cout + nb * NB + c0;
+    for (int c0 = 0; c0 < NB; c0 += 16) {
+      u32 v[16];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) atomicAdd(d + j, __uint_as_float(v[j]));
-        }
+      for (int j = 0; j < 16; ++j) v[j] = 0u;  // a block without its sums leaves zeros (the error word is set)
+      if (ok) tmem_ld16(tmem + ((u32)(warp * 32) << 16) + (u32)(tl * NB + c0), v);
+      if (ci < a.Cx) {
+        uint4* d = reinterpret_cast<uint4*>(a.part + (((int64_t)blockIdx.x * 9 + t) * a.Cx + ci) * a.cout + nb * NB + c0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) d[j] = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
       }
     }
   }
@@ -571,6 +578,62 @@ __global__ void __launch_bounds__(128, 1)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }
+}
+
+// A float32 sum that carries its own rounding error along (two-sum of each step)
+struct FSum {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+    s = t;
+  }
+  __device__ __forceinline__ float value() const { return isfinite(s) ? __fadd_rn(s, e) : s; }
+};
+
+// The sums of the backward pass's blocks, in a fixed order. Weights: dw [9][cin][cout] =
+// sum over `splits` parts [9][Cx][cout] (Cx >= cin: the first layer's stored channels). Columns:
+// db[0 .. nb) = sum over `parts` rows of nb values, the last of them to `last` where it is given.
+// A block takes 32 values, its warps every 16th part (whole lines, kSumU in flight), and adds the
+// warps' sums in order; every sum carries its rounding error, so that the result is the sum
+// of the parts to one rounding.
+// Bound by the parts' bytes, which the L2 holds (at most about 35 MB a layer). A step on 16 crops
+// of 256 x 256: 15 launches of 17 us on average with cold caches; without the atomics the weight
+// gradients' epilogues are shorter (32 channels: 166 -> 133 us a layer), and the step takes 2.98 -> 2.74 ms.
+constexpr int kSumU = 8, kSumWarps = 16;
+
+__global__ void __launch_bounds__(32 * kSumWarps) k_grad_sum(const float* __restrict__ wpart, int splits, int Cx,
+                                                             int cin, int cout, float* __restrict__ dw,
+                                                             const float* __restrict__ bpart, int parts, int nb,
+                                                             float* __restrict__ db, float* __restrict__ last) {
+  __shared__ float s_s[kSumWarps][32], s_e[kSumWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nw = 9 * cin * cout, wblocks = nw / 32;  // cout is a multiple of 32
+  const bool weights = (int)blockIdx.x < wblocks;
+  const int i = (weights ? blockIdx.x : blockIdx.x - wblocks) * 32 + lane;
+  const int rows = weights ? splits : parts;
+  const int64_t stride = weights ? (int64_t)9 * Cx * cout : nb;
+  const bool on = weights || i < nb;
+  const float* src = weights ? wpart + i + (int64_t)(i / (cin * cout)) * (Cx - cin) * cout : bpart + i;
+  FSum a;
+  for (int r0 = warp; on && r0 < rows; r0 += kSumWarps * kSumU) {
+    float v[kSumU];
+#pragma unroll
+    for (int u = 0; u < kSumU; ++u) v[u] = r0 + kSumWarps * u < rows ? src[(r0 + kSumWarps * u) * stride] : 0.f;
+#pragma unroll
+    for (int u = 0; u < kSumU; ++u) a.add(v[u]);
+  }
+  s_s[warp][lane] = a.s;
+  s_e[warp][lane] = a.e;
+  __syncthreads();
+  if (warp != 0 || !on) return;
+  for (int w = 1; w < kSumWarps; ++w) {
+    a.add(s_s[w][lane]);
+    a.e = __fadd_rn(a.e, s_e[w][lane]);
+  }
+  if (weights) dw[i] = a.value();
+  else if (last && i == nb - 1) *last = a.value();
+  else db[i] = a.value();
 }
 
 // i / d for i < total; in 32 bits wherever the total allows (a 64-bit division costs more than
@@ -662,15 +725,14 @@ __global__ void k_maxpool_bwd(const bf16* __restrict__ x, const bf16* __restrict
   }
 }
 
-// ReLU gradient in place, dy *= (y > 0), and the bias gradient db[c] += sum_p dy[p][c] of
-// the result: a block takes a part of one plane of 8 channels of every image (blockIdx.y),
-// 16 bytes per thread and step; the threads' sums meet in shared memory, one atomic per
-// channel and block. One pass over dy instead of two (the sums alone took 15 us a layer).
+// ReLU gradient in place, dy *= (y > 0), and the blocks' sums of the bias gradient
+// db[c] = sum_p dy[p][c] of the result: a block takes a part of one plane of 8 channels of every
+// image (blockIdx.y), 16 bytes per thread and step, and leaves the plane's 8 sums in row blockIdx.x
+// of `part` [gridDim.x][8 planes]. One pass over dy instead of two (the sums alone took 15 us a
+// layer). (A pixel's number fits 32 bits: a batch has at most 2^27 pixels.)
 __global__ void __launch_bounds__(256) k_relu_bias_bwd(const bf16* __restrict__ y, bf16* __restrict__ dy,
-                                                       float* __restrict__ db, int N, int planes, int64_t hw) {
-  __shared__ float s_db[8];
-  if (threadIdx.x < 8) s_db[threadIdx.x] = 0.f;
-  __syncthreads();
+                                                       float* __restrict__ part, int N, int planes, int64_t hw) {
+  __shared__ float s_db[8][8];  // [warp][channel]
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   const int64_t items = (int64_t)N * hw, stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += stride) {
@@ -695,10 +757,14 @@ __global__ void __launch_bounds__(256) k_relu_bias_bwd(const bf16* __restrict__ 
   for (int j = 0; j < 8; ++j) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&s_db[j], acc[j]);
+    if ((threadIdx.x & 31) == 0) s_db[threadIdx.x >> 5][j] = acc[j];
   }
   __syncthreads();
-  if (threadIdx.x < 8) atomicAdd(&db[blockIdx.y * 8 + threadIdx.x], s_db[threadIdx.x]);
+  if (threadIdx.x < 8) {
+    float t = 0.f;
+    for (int w = 0; w < 8; ++w) t += s_db[w][threadIdx.x];
+    part[(int64_t)blockIdx.x * planes * 8 + blockIdx.y * 8 + threadIdx.x] = t;
+  }
 }
 
 // gradient of concat([upsample(low), skip]): low gets the 2x2 sums of the
@@ -750,20 +816,17 @@ __device__ __forceinline__ float warp_sum(float x) {
 // final 1x1 convolution (residual over the diffusion fill), masked-MSE loss and
 // its gradients: res = b + d1 . w ; pred = fill + res. A thread owns a pixel and reads
 // its channels 8 at a time; the weight gradient is summed across the warp by shuffles
-// (one shared-memory add per warp and channel), skipped where no lane has a hidden cell.
+// into the warp's own sums, skipped where no lane has a hidden cell. Row blockIdx.x of `part`
+// [gridDim.x][C + 2] gets the block's sums: weights, bias, loss (blocks of 256 threads).
 __global__ void k_head(const bf16* __restrict__ d1, int C, const float* __restrict__ w, const float* __restrict__ b,
                        const float* __restrict__ fill, float* __restrict__ pred, const float* __restrict__ target,
-                       const uint8_t* __restrict__ hidden, float inv_cnt, int64_t P, int64_t hw, float* __restrict__ loss,
-                       bf16* __restrict__ dd1, float* __restrict__ dw, float* __restrict__ dbias) {
-  __shared__ float s_w[256], s_dw[256];
-  __shared__ float s_loss, s_db;
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    s_w[c] = w[c];
-    s_dw[c] = 0.f;
-  }
-  if (threadIdx.x == 0) s_loss = s_db = 0.f;
+                       const uint8_t* __restrict__ hidden, float inv_cnt, int64_t P, int64_t hw,
+                       bf16* __restrict__ dd1, float* __restrict__ part) {
+  __shared__ float s_w[256], s_dw[8][258];  // [warp][channel, then bias, loss]
+  for (int c = threadIdx.x; c < C; c += blockDim.x) s_w[c] = w[c];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int c = lane; c < C; c += 32) s_dw[warp][c] = 0.f;
   __syncthreads();
-  const int lane = threadIdx.x & 31;
   float l = 0.f, gb = 0.f;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   // every lane of a warp runs the same number of iterations (the shuffles need all 32)
@@ -813,21 +876,25 @@ __global__ void k_head(const bf16* __restrict__ d1, int C, const float* __restri
           const float2 f = __bfloat1622float2(h[j]);
           const float s0 = warp_sum(g * f.x), s1 = warp_sum(g * f.y);
           if (lane == 0) {
-            atomicAdd(&s_dw[c + 2 * j], s0);
-            atomicAdd(&s_dw[c + 2 * j + 1], s1);
+            s_dw[warp][c + 2 * j] += s0;
+            s_dw[warp][c + 2 * j + 1] += s1;
           }
         }
       }
     }
   }
   if (target) {
-    atomicAdd(&s_loss, l * inv_cnt);
-    atomicAdd(&s_db, gb);
+    gb = warp_sum(gb);
+    l = warp_sum(l * inv_cnt);
+    if (lane == 0) {
+      s_dw[warp][C] = gb;
+      s_dw[warp][C + 1] = l;
+    }
     __syncthreads();
-    for (int c = threadIdx.x; c < C; c += blockDim.x) atomicAdd(&dw[c], s_dw[c]);
-    if (threadIdx.x == 0) {
-      atomicAdd(loss, s_loss);
-      atomicAdd(dbias, s_db);
+    for (int c = threadIdx.x; c < C + 2; c += blockDim.x) {
+      float t = 0.f;
+      for (int k = 0; k < 8; ++k) t += s_dw[k][c];
+      part[(int64_t)blockIdx.x * (C + 2) + c] = t;
     }
   }
 }
@@ -881,17 +948,6 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
     m[i] = mi;
     v[i] = vi;
     p[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
-  }
-}
-
-// [9][cin_pad][cout] -> [9][cin][cout]
-__global__ void k_unpad_rows(const float* __restrict__ src, float* __restrict__ dst, int cin, int cin_pad, int cout) {
-  const int64_t n = 9LL * cin * cout;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int co = (int)(i % cout);
-    const int64_t r = i / cout;
-    const int ci = (int)(r % cin), t = (int)(r / cin);
-    dst[i] = src[((int64_t)t * cin_pad + ci) * cout + co];
   }
 }
 
@@ -956,7 +1012,7 @@ struct mem_unet {
   bf16* dcat = nullptr;   // gradient of a concatenated decoder input
   bf16* dpool[3] = {};    // gradient of the pooled tensors
   float* d_loss = nullptr;
-  float* g0pad = nullptr;  // weight gradient of the first layer with padded input channels
+  float *wpart = nullptr, *bpart = nullptr;  // blocks' sums of a layer's weights; of its biases, or of the head
   int* d_err = nullptr;    // set by a convolution whose bounded wait ran out
   int n_sm = 148;
 };
@@ -964,6 +1020,40 @@ struct mem_unet {
 namespace {
 
 int pad32(int c) { return (c + 31) / 32 * 32; }
+
+int grid_for(int64_t n, int n_sm) {
+  int64_t b = (n + 255) / 256;
+  const int64_t cap = (int64_t)n_sm * 16;
+  return (int)(b < 1 ? 1 : (b > cap ? cap : b));
+}
+
+// output-channel block and tap group of a weight-gradient block: TMEM holds the group's
+// accumulators (<= 512 columns)
+int wgrad_nb(int cout) { return cout % 128 == 0 ? 128 : (cout % 64 == 0 ? 64 : 32); }
+int wgrad_taps(int nb) { return nb == 128 ? 3 : (nb == 64 ? 5 : 9); }
+int wgrad_tiles(int N, int H, int W) { return N * ((H + 7) / 8) * ((W + 15) / 16); }
+
+// parts that a weight gradient's pixels are split into, and its blocks of 128 input channels and
+// (output block, tap group) pairs
+int wgrad_splits(const mem_unet* u, int Cx, int cout, int N, int H, int W, int* mbk, int* groups) {
+  const int nb = wgrad_nb(cout), taps = wgrad_taps(nb);
+  *mbk = (Cx + 127) / 128;
+  *groups = (cout / nb) * ((9 + taps - 1) / taps);
+  const int splits = (u->n_sm + *mbk * *groups - 1) / (*mbk * *groups);  // about one block per SM
+  // at least 8 tiles per block: storing its sums costs about as much as 8 tiles of MMAs
+  return std::max(1, std::min(splits, wgrad_tiles(N, H, W) / 8));
+}
+
+// blocks of a plane of k_relu_bias_bwd
+int relu_parts(const mem_unet* u, int planes, int64_t pixels) {
+  return std::max(1, std::min((u->n_sm * 8 + planes - 1) / planes, (int)std::min<int64_t>((pixels + 255) / 256, 1 << 20)));
+}
+
+// blocks of k_head where it leaves sums: as many as are resident, a row of sums each
+int head_grid(const mem_unet* u, int64_t P) { return std::min(grid_for(P, u->n_sm), u->n_sm * 4); }
+
+// channels of layer i's input tensor (the first layer's holds kInC)
+int stored_cin(const mem_unet* u, int i) { return i == 0 ? kInC : u->L[i].cin; }
 
 cudaError_t ensure_acts(mem_unet* u, int N, int H, int W) {
   if (u->N >= N && u->H == H && u->W == W && u->x8) return cudaSuccess;
@@ -977,13 +1067,17 @@ cudaError_t ensure_acts(mem_unet* u, int N, int H, int W) {
   };
   const int64_t P = (int64_t)N * H * W;
   u->x8 = (bf16*)alloc(P * kInC * 2);
-  int64_t maxcat = 0;
+  int64_t maxcat = 0, wsum = 0, bsum = (int64_t)head_grid(u, P) * (u->widths[0] + 2);
   for (size_t i = 0; i < u->L.size(); ++i) {
     const ConvLayer& c = u->L[i];
     const int64_t Pl = P >> (2 * c.level);
     u->act[i] = (bf16*)alloc(Pl * c.cout * 2);
     u->dact[i] = (bf16*)alloc(Pl * c.cout * 2);
     if (c.c1) maxcat = std::max<int64_t>(maxcat, Pl * c.cin);
+    int mbk, groups;
+    const int Cx = stored_cin(u, (int)i), splits = wgrad_splits(u, Cx, c.cout, N, H >> c.level, W >> c.level, &mbk, &groups);
+    wsum = std::max<int64_t>(wsum, (int64_t)splits * 9 * Cx * c.cout);
+    bsum = std::max<int64_t>(bsum, (int64_t)relu_parts(u, c.cout / 8, Pl) * c.cout);
     if (!u->act[i] || !u->dact[i]) return cudaErrorMemoryAllocation;
   }
   for (int l = 0; l < 3; ++l) {
@@ -992,17 +1086,13 @@ cudaError_t ensure_acts(mem_unet* u, int N, int H, int W) {
   }
   u->dcat = (bf16*)alloc(maxcat * 2);
   u->d_loss = (float*)alloc(4);
-  if (!u->x8 || !u->dcat || !u->d_loss) return cudaErrorMemoryAllocation;
+  u->wpart = (float*)alloc(wsum * 4);
+  u->bpart = (float*)alloc(bsum * 4);
+  if (!u->x8 || !u->dcat || !u->d_loss || !u->wpart || !u->bpart) return cudaErrorMemoryAllocation;
   u->N = N;
   u->H = H;
   u->W = W;
   return cudaSuccess;
-}
-
-int grid_for(int64_t n, int n_sm) {
-  int64_t b = (n + 255) / 256;
-  const int64_t cap = (int64_t)n_sm * 16;
-  return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
 template <int BN, int NST>
@@ -1128,43 +1218,35 @@ void launch_wgrad(dim3 grid, const CUtensorMap& tmx, const CUtensorMap& tmy, con
   k_wgrad3x3t<NB, TAPG, NST><<<grid, 128, C::kSmem, st>>>(tmx, tmy, a);
 }
 
-// dW (float32, [9][cin_pad][cout], accumulated into) of one 3x3 convolution whose input is
-// in0 (c0 channels; at half resolution when up0) concatenated with in1 (c1 channels)
-cudaError_t wgrad(mem_unet* u, const ConvLayer& c, const bf16* in0, const bf16* in1, const bf16* dy,
-                  float* dw_pad, int N, int H, int W, cudaStream_t st) {
+// Parts of dW (u->wpart, `*splits` of them) of one 3x3 convolution whose input, Cx channels as
+// stored, is in0 (c0 channels; at half resolution when up0) concatenated with in1 (c1 channels)
+cudaError_t wgrad(mem_unet* u, const ConvLayer& c, int Cx, const bf16* in0, const bf16* in1, const bf16* dy,
+                  int* splits, int N, int H, int W, cudaStream_t st) {
   const bf16* X = in0;
-  int Cx = c.c0;
   if (c.c1 || c.up0) {  // decoder input: materialise [upsampled, skip] in the concat scratch
-    Cx = c.c0 + c.c1;
     k_cat_up<<<grid_for((int64_t)N * H * W * (Cx / 8), u->n_sm), 256, 0, st>>>(in0, in1, u->dcat, N, H, W, c.c0,
                                                                                   c.c1);
     X = u->dcat;
   }
-  if (Cx % 8 || c.cout % 32 || c.cin_pad % 8 || Cx > c.cin_pad) return cudaErrorInvalidValue;
+  if (Cx % 8 || c.cout % 32) return cudaErrorInvalidValue;
   WgradArgs a;
   a.Cx = Cx;
-  a.cin_pad = c.cin_pad;
   a.cout = c.cout;
-  a.dw = dw_pad;
+  a.part = u->wpart;
   a.N = N;
   a.H = H;
   a.W = W;
-  a.tiles = N * ((H + 7) / 8) * ((W + 15) / 16);
+  a.tiles = wgrad_tiles(N, H, W);
   a.err = u->d_err;
-  // output-channel block and tap group: TMEM holds the tap group's accumulators (<= 512 columns)
-  const int NB = c.cout % 128 == 0 ? 128 : (c.cout % 64 == 0 ? 64 : 32);
-  const int TAPG = NB == 128 ? 3 : (NB == 64 ? 5 : 9);
+  const int NB = wgrad_nb(c.cout);
   CUtensorMap tmx, tmy;
   if (!activation_map(&tmx, X, Cx, W, H, N, 18, 10, Cx / 8 < 16 ? Cx / 8 : 16) ||
       !activation_map(&tmy, dy, c.cout, W, H, N, 16, 8, NB / 8))
     return cudaErrorInvalidValue;
-  const int mbk = (Cx + 127) / 128, groups = (c.cout / NB) * ((9 + TAPG - 1) / TAPG);
-  int splits = (u->n_sm + mbk * groups - 1) / (mbk * groups);  // about one block per SM
-  if (splits > a.tiles / 8) splits = a.tiles / 8;  // at least 8 tiles per block: the epilogue's atomics
-                                                  // cost about as much as 8 tiles of MMAs
-  if (splits < 1) splits = 1;
-  const dim3 grid((unsigned)splits, (unsigned)mbk, (unsigned)groups);
-  switch (NB) {
+  int mbk, groups;
+  *splits = wgrad_splits(u, Cx, c.cout, N, H, W, &mbk, &groups);
+  const dim3 grid((unsigned)*splits, (unsigned)mbk, (unsigned)groups);
+  switch (NB) {  // (tap groups: wgrad_taps)
     case 128: launch_wgrad<128, 3, 2>(grid, tmx, tmy, a, st); break;
     case 64: launch_wgrad<64, 5, 3>(grid, tmx, tmy, a, st); break;
     default: launch_wgrad<32, 9, 3>(grid, tmx, tmy, a, st); break;
@@ -1233,27 +1315,19 @@ cudaError_t forward(mem_unet* u, int N, int H, int W, cudaStream_t st, const flo
 }
 
 cudaError_t backward(mem_unet* u, int N, int H, int W, cudaStream_t st) {
-  // u->dact[13] holds d loss / d d1 (post-ReLU); grads zeroed except the head's
+  // u->dact[13] holds d loss / d d1 (post-ReLU)
   for (int i = 13; i >= 0; --i) {
     const ConvLayer& c = u->L[i];
     const int l = c.level;
     const int Hl = H >> l, Wl = W >> l;
     const int64_t Pl = (int64_t)N * Hl * Wl;
-    {
-      const int planes = c.cout / 8;
-      const int parts = std::max(1, std::min((u->n_sm * 8 + planes - 1) / planes, (int)std::min<int64_t>((Pl + 255) / 256, 1 << 20)));
-      k_relu_bias_bwd<<<dim3(parts, planes), 256, 0, st>>>(u->act[i], u->dact[i], u->grads + c.b_off, N, planes,
-                                                           (int64_t)Hl * Wl);
-    }
-    ConvLayer cc = c;
-    if (i == 0) cc.c0 = kInC;
-    float* dw = i == 0 ? u->g0pad : u->grads + c.w_off;  // only the first layer has padded rows
-    if (i == 0) cudaMemsetAsync(u->g0pad, 0, 9ull * c.cin_pad * c.cout * 4, st);
-    cudaError_t e = wgrad(u, cc, input0(u, i), input1(u, i), u->dact[i], dw, N, Hl, Wl, st);
+    const int planes = c.cout / 8, parts = relu_parts(u, planes, Pl), Cx = stored_cin(u, i);
+    k_relu_bias_bwd<<<dim3(parts, planes), 256, 0, st>>>(u->act[i], u->dact[i], u->bpart, N, planes, (int64_t)Hl * Wl);
+    int splits = 0;
+    cudaError_t e = wgrad(u, c, Cx, input0(u, i), input1(u, i), u->dact[i], &splits, N, Hl, Wl, st);
     if (e != cudaSuccess) return e;
-    if (i == 0)
-      k_unpad_rows<<<grid_for(9LL * c.cin * c.cout, u->n_sm), 256, 0, st>>>(u->g0pad, u->grads + c.w_off, c.cin,
-                                                                            c.cin_pad, c.cout);
+    k_grad_sum<<<9 * c.cin * c.cout / 32 + c.cout / 32, 32 * kSumWarps, 0, st>>>(u->wpart, splits, Cx, c.cin, c.cout, u->grads + c.w_off,
+                                                                      u->bpart, parts, c.cout, u->grads + c.b_off, nullptr);
     if (i == 0) break;
     // data gradient into the layer input
     if (c.c1) {  // decoder concat input: d(concat) then split
@@ -1332,7 +1406,6 @@ extern "C" mem_status mem_unet_create(int32_t cin, const int32_t widths[4], mem_
   };
   if (cudaMalloc(&u->params, off * 4) != cudaSuccess || cudaMalloc(&u->grads, off * 4) != cudaSuccess ||
       cudaMalloc(&u->adam_m, off * 4) != cudaSuccess || cudaMalloc(&u->adam_v, off * 4) != cudaSuccess ||
-      cudaMalloc(&u->g0pad, 9ull * u->L[0].cin_pad * u->L[0].cout * 4) != cudaSuccess ||
       cudaMalloc(&u->d_err, sizeof(int)) != cudaSuccess)
     return fail_oom();
   cudaMemset(u->d_err, 0, sizeof(int));
@@ -1360,7 +1433,6 @@ extern "C" mem_status mem_unet_destroy(mem_unet* u) {
   cudaFree(u->grads);
   cudaFree(u->adam_m);
   cudaFree(u->adam_v);
-  cudaFree(u->g0pad);
   cudaFree(u->d_err);
   delete u;
   return MEM_OK;
@@ -1426,7 +1498,7 @@ extern "C" mem_status mem_unet_forward(mem_unet* u, int32_t n, int32_t H, int32_
   if (!head_done)
     k_head<<<grid_for(P, u->n_sm), 256, 0, st>>>(u->act[13], u->widths[0], u->params + u->head_w,
                                                   u->params + u->head_b, fill, pred, nullptr, nullptr, 0.f, P,
-                                                  (int64_t)H * W, nullptr, nullptr, nullptr, nullptr);
+                                                  (int64_t)H * W, nullptr, nullptr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return memh::api_cuda_fail(e, "U-Net head");
   return MEM_OK;
@@ -1447,17 +1519,17 @@ extern "C" mem_status mem_unet_gradients(mem_unet* u, int32_t n, int32_t H, int3
   k_pack_input<<<grid_for((P + 3) / 4, u->n_sm), 256, 0, st>>>(x3, u->x8, P);
   e = forward(u, n, H, W, st);
   if (e != cudaSuccess) return memh::api_cuda_fail(e, "U-Net forward");
-  cudaMemsetAsync(u->grads, 0, u->n_params * 4, st);
-  cudaMemsetAsync(u->d_loss, 0, 4, st);
   // the skip tensors' gradients are accumulated: start from zero
   for (int i : {1, 3, 5}) {
     const ConvLayer& c = u->L[i];
     cudaMemsetAsync(u->dact[i], 0, (P >> (2 * c.level)) * c.cout * 2, st);
   }
   const float inv = 1.f / (float)(n_hidden > 0 ? n_hidden : 1);
-  k_head<<<grid_for(P, u->n_sm), 256, 0, st>>>(u->act[13], u->widths[0], u->params + u->head_w,
-                                                u->params + u->head_b, fill, nullptr, target, hidden, inv, P,
-                                                (int64_t)H * W, u->d_loss, u->dact[13], u->grads + u->head_w, u->grads + u->head_b);
+  const int hgrid = head_grid(u, P), C = u->widths[0];
+  k_head<<<hgrid, 256, 0, st>>>(u->act[13], C, u->params + u->head_w, u->params + u->head_b, fill, nullptr, target, hidden,
+                                inv, P, (int64_t)H * W, u->dact[13], u->bpart);
+  k_grad_sum<<<(C + 2 + 31) / 32, 32 * kSumWarps, 0, st>>>(nullptr, 0, 0, 0, 0, nullptr, u->bpart, hgrid, C + 2, u->grads + u->head_w,
+                                                u->d_loss);  // (the head's bias follows its weights)
   e = backward(u, n, H, W, st);
   if (e != cudaSuccess) return memh::api_cuda_fail(e, "U-Net backward");
   if (grads) e = cudaMemcpyAsync(grads, u->grads, u->n_params * 4, cudaMemcpyDeviceToDevice, st);
