@@ -1056,12 +1056,21 @@ int head_grid(const mem_unet* u, int64_t P) { return std::min(grid_for(P, u->n_s
 int stored_cin(const mem_unet* u, int i) { return i == 0 ? kInC : u->L[i].cin; }
 
 cudaError_t ensure_acts(mem_unet* u, int N, int H, int W) {
-  if (u->N >= N && u->H == H && u->W == W && u->x8) return cudaSuccess;
-  for (void* p : u->bufs) cudaFree(p);
-  u->bufs.clear();
+  if (u->N >= N && u->H == H && u->W == W) return cudaSuccess;
+  auto release = [&]() {
+    for (void* p : u->bufs) cudaFree(p);
+    u->bufs.clear();
+    u->N = u->H = u->W = 0;  // no shape has its buffers until all of them are there
+  };
+  release();
+  bool ok = true;
   auto alloc = [&](size_t bytes) -> void* {
     void* p = nullptr;
-    if (cudaMalloc(&p, bytes ? bytes : 16) != cudaSuccess) return nullptr;
+    if (ok && cudaMalloc(&p, bytes ? bytes : 16) != cudaSuccess) {
+      cudaGetLastError();  // returned below: not left for the next launch's check
+      ok = false;
+    }
+    if (!ok) return nullptr;
     u->bufs.push_back(p);
     return p;
   };
@@ -1078,7 +1087,6 @@ cudaError_t ensure_acts(mem_unet* u, int N, int H, int W) {
     const int Cx = stored_cin(u, (int)i), splits = wgrad_splits(u, Cx, c.cout, N, H >> c.level, W >> c.level, &mbk, &groups);
     wsum = std::max<int64_t>(wsum, (int64_t)splits * 9 * Cx * c.cout);
     bsum = std::max<int64_t>(bsum, (int64_t)relu_parts(u, c.cout / 8, Pl) * c.cout);
-    if (!u->act[i] || !u->dact[i]) return cudaErrorMemoryAllocation;
   }
   for (int l = 0; l < 3; ++l) {
     u->pool[l] = (bf16*)alloc((P >> (2 * (l + 1))) * u->widths[l] * 2);
@@ -1088,7 +1096,10 @@ cudaError_t ensure_acts(mem_unet* u, int N, int H, int W) {
   u->d_loss = (float*)alloc(4);
   u->wpart = (float*)alloc(wsum * 4);
   u->bpart = (float*)alloc(bsum * 4);
-  if (!u->x8 || !u->dcat || !u->d_loss || !u->wpart || !u->bpart) return cudaErrorMemoryAllocation;
+  if (!ok) {
+    release();
+    return cudaErrorMemoryAllocation;
+  }
   u->N = N;
   u->H = H;
   u->W = W;

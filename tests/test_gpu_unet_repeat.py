@@ -52,3 +52,27 @@ def test_gradients_match_oracle_over_many_tiles(torch, widths, N, H, W):  # noqa
     bad = [(n, rel, c, floor[n]) for n, rel, c in _grad_errors(g, go)
            if not (rel <= 2e-2 or c >= 0.999 or (floor[n] > 2e-2 and rel <= 3 * floor[n]))]
     assert not bad, bad
+
+
+def test_a_batch_that_does_not_fit_leaves_the_network_usable(torch):  # noqa: F811
+    """2^27 cells at 256 channels need several times the device's memory: refused as out of memory,
+    after which the shape that had its buffers before gets new ones and the same results."""
+    from paper_2309_16818_gb300 import mem as M
+    from paper_2309_16818_gb300.inpaint import init_params
+    widths = (256, 256, 256, 256)
+    if torch.cuda.get_device_properties(0).total_memory > 400 << 30:
+        pytest.skip("such a batch may fit this device")
+    net = M.UNet(3, widths)
+    net.set_params(torch.from_numpy(init_params(1, 3, widths, out_scale=1.0)).cuda())
+    rng = np.random.default_rng(5)
+    x3 = torch.from_numpy(rng.normal(size=(2, 32, 24, 3)).astype(np.float32)).cuda()
+    fill = torch.from_numpy(rng.normal(size=(2, 32, 24)).astype(np.float32)).cuda()
+    before = net.forward(x3, fill)
+    n, S = 8, 4096
+    big = torch.zeros((1, 1, 1, 3), device="cuda").expand(n, S, S, 3)  # (never read: refused before any launch)
+    with pytest.raises(M.MemError, match="memory"):
+        net.forward(big, fill, out=fill)
+    again = net.forward(x3, fill)
+    net.check()
+    assert torch.equal(before, again)
+    net.close()
