@@ -307,7 +307,7 @@ def run_ours(args):
         # layer of every touched cell read and written
         "fuse_tiles": kept * (4 + 4 + 12 + payload) + cells * cb,
     }
-    # the warp fuse kernel fuses the runs that cross tiles itself (no k_fuse_cross launch)
+    # (launches of the crossing-run and move kernels: as profiled)
     launches = {"key": K, "radix_sort": K * P, "fuse_tiles": K, "fuse_cross": prof["fuse_cross"][1],
                 "move": prof["move"][1]}
     kern = {}

@@ -3,8 +3,8 @@
 // i.e. the discrete Laplace equation with the known cells as boundary values.
 //
 // A crop that fits the shared memory of a cluster of up to 8 CTAs is solved by
-// k_inpaint_sor_cluster (its rows split over the cluster, boundary rows read
-// from the neighbours' shared memory); larger crops by k_inpaint_sor, one
+// k_inpaint_sor_cluster (its rows split over the cluster, boundary rows written
+// into the neighbours' shared memory); larger crops by k_inpaint_sor, one
 // thread block per crop working in global memory (L2-resident).
 // Unknown cells start from the mean of the crop's known cells; the sweeps stop
 // when the largest update of a full sweep falls below `tol` or after

@@ -464,8 +464,9 @@ constexpr int kSegMax = 32;     // segments of a tile per walk
 constexpr int kStageU = 6;      // staging chunks in flight per thread
 constexpr int kStageV = 5;      // float4 row loads in flight per thread (warp fuse kernel)
 constexpr int kApplyU = 4;      // rule tasks in flight per thread
-constexpr int kWarpBlocks = 6;  // resident CTAs per SM of the warp fuse kernel (80 registers; 7: 48.6, 8: 48.1 us
-                                // against 43.4, from spills)
+constexpr int kWarpBlocks = 6;  // resident CTAs per SM of the warp fuse kernel: 80 registers, which the variants of one
+                                // round fit (7: 48.6, 8: 48.1 us against 43.4, from spills) and those of several rounds
+                                // miss by 20 to 36 bytes of spill stores (three rounds: 87.2 us, 92.8 and 81.2 with 7 and 8)
 constexpr int kCrossU = 8;      // slot pieces in flight per lane (runs crossing tiles)
 constexpr u32 kBitHead = 1u;    // slot bits: the run begins in the tile
 constexpr u32 kBitEnd = 2u;     //            the run ends in the tile
@@ -1334,7 +1335,8 @@ __device__ __forceinline__ void cross_run(const MapDev& md, const LayerDev* sL, 
 
 // ---------------------------------------------------------------------------
 // 4b. the same fusion with the per-cell sums taken by warps, for calls that fit a
-//     FusePlan (up to 192 summed columns in rounds of 32; wider calls go to
+//     FusePlan (six rounds of at most 32 summed columns, 16 staged segments, 40 rules:
+//     192 columns at most, fewer where sources split unevenly; others go to
 //     k_fuse_tiles). A warp holds 32 consecutive points of the tile, one per lane.
 //     Per round: each lane stages its point's channels in its own shared-memory row
 //     (round 0 adds the height sums after the gate); lane c walks column c down the

@@ -179,6 +179,10 @@ __host__ __device__ inline int conv_bn(int cout) { return cout % 128 == 0 ? 128 
 // arrivals + the copied bytes), slot empty (MMA commit), half-resolution
 // staging full (its bytes), accumulator full (MMA commit), accumulator empty
 // (128 epilogue arrivals). Every wait is bounded.
+//
+// BN = 32 runs four blocks per SM (TMEM), which leaves 64 registers a thread: the 64-bit strides
+// between the output's planes spill 20 bytes of stores and 24 of loads there, and the kernel takes
+// 585 us on average over the 256-crop inference's four such layers (634 without planes or spills).
 constexpr int kTY = 16, kTX = 16;              // output tile
 constexpr int kHY = kTY + 2, kHX = kTX + 2;    // input halo
 constexpr int kPlane = kHY * kHX * 16;         // bytes of one 8-channel halo plane (5184)
